@@ -92,12 +92,12 @@ __device__ __forceinline__ double seed_square(double t) {
 }
 
 // For t with at most 21 significant bits (the low 32 bits of its encoding
-// zero, as the MUFU seeds are) and k >= 0: t^2
+// zero, as the MUFU seeds are) and any k: t^2
 // exactly and k t^3 correctly rounded (ties away from zero) by integer
 // arithmetic.  The 53-bit significand of k times m^3 (63 bits, exact) is a
 // 116-bit product; its top 64 bits come from one 64 x 64 high multiply
 // (the low bits can only matter for an exact tie) and are rounded to 53.
-// k = 0 (or subnormal) gives 0.  Returns false (kt3 unspecified) when t is
+// k = 0 (or subnormal) gives 0; a negative k (a backward step's dt G m) its sign.  Returns false (kt3 unspecified) when t is
 // outside [2^-300, 2^300] or not normal, k is not finite, or k t^3 leaves
 // the normal range.
 __device__ __forceinline__ bool seed_square_kcube(double t, double k, double& t2, double& kt3) {
@@ -115,7 +115,8 @@ __device__ __forceinline__ bool seed_square_kcube(double t, double k, double& t2
     const int sh = 11 - __clzll(p);                               // leading bit at 52 + sh
     const unsigned long long q = ((p >> (sh - 1)) + 1) >> 1;      // 53 bits, rounded
     const int be = sh + ek + 3 * et - 3077;                       // biased exponent of k t^3
-    kt3 = (ek == 0) ? 0.0 : __longlong_as_double(((long long)(be - 1) << 52) + (long long)q);
+    kt3 = (ek == 0) ? 0.0
+                    : __longlong_as_double((((long long)(be - 1) << 52) + (long long)q) | (kb & (long long)(1ull << 63)));
     return (unsigned)(et - 723) <= 600u && ek != 0x7FF && (ek == 0 || (unsigned)(be - 1) < 2045u);
 }
 

@@ -181,6 +181,24 @@ def test_ragged_particle_counts(G, orc, n):
     assert rep["n"] == n
 
 
+def test_backward_steps_undo_forward_ones(G):
+    """The map is time-reversible: steps of -dt from the state that steps of dt reached lead back to the
+    start, to the rounding of both runs.  A kick with the wrong sign of dt misses by 1e-2."""
+    w = gi.make("tiny", n=128)
+    n_steps = 200
+    sim = G.Simulation(w["star_mass"], w["planets"], w["particles"], w["dt"])
+    sim.advance(n_steps)
+    there, pl = sim.read(), sim.planets()[0]
+    sim.close()
+    assert there["alive"].all()
+    back = G.Simulation(w["star_mass"], pl, there["state"], -w["dt"])
+    back.advance(n_steps)
+    got = back.read()["state"]
+    back.close()
+    # ~10 ulp of the orbit per step each way, phase growing as n^1.5 (see parity.state_tol)
+    assert parity.rel_err(got, w["particles"]).max() < 1e-11
+
+
 def test_zero_particles(G):
     w = gi.make("tiny", n=0)
     g = run_gpu(G, w, 50)
