@@ -144,7 +144,7 @@ int glisse_create(glisse_ctx** out, double star_mass, const double* planets, int
  * of the chunk waits for the whole planet chunk instead.  A call longer than a
  * few chunks lets the planets run ahead of the particles up to its last chunk:
  * the planet-log buffers then grow (once, kept until glisse_destroy) to up to
- * 512 MB, (C + 1) x (4 (N_p + 1) + 6 N_p) doubles per chunk held.
+ * 512 MB, (C + 1) x (8 (N_p + 1) + 6 N_p) doubles per chunk held.
  * Splitting a run into calls changes nothing: advance(a) then advance(b) gives
  * bit for bit what advance(a + b) gives.  Between calls the device keeps each
  * live particle's velocity with the next step's opening half kick already

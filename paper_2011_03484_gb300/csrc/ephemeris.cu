@@ -24,8 +24,19 @@
 //   S_k = sum_{i > k} m_i ghat_i
 #include "glisse_internal.h"
 #include "kepler.cuh"
+#include "split_math.cuh"
 
 namespace glisse {
+
+// One log record: (x, y, z) as doubles, (sx, sy, sz) as pairs (the same vector, or dt times it).
+__device__ __forceinline__ void store_rec(double* __restrict__ rec, double x, double y, double z, double sx, double sy,
+                                          double sz) {
+    const F2 a = f2_split(sx), b = f2_split(sy), c = f2_split(sz);
+    reinterpret_cast<double2*>(rec)[0] = make_double2(x, y);
+    reinterpret_cast<double2*>(rec)[1] = make_double2(z, 0.0);
+    reinterpret_cast<float4*>(rec + kRecSplit)[0] = make_float4(a.h, b.h, c.h, a.l);
+    reinterpret_cast<float4*>(rec + kRecSplit)[1] = make_float4(b.l, c.l, 0.0f, 0.0f);
+}
 
 // Scans over the first n lanes (n <= 32, warp-uniform).  Lanes >= n must hold 0.
 // exclusive prefix: sum over lanes k < lane
@@ -315,7 +326,7 @@ __device__ __forceinline__ void eph_dynamics(const PlanetConsts& pc, double* jac
 // progress (optional, host-mapped): after every kProgressEvery-th step and the last, the
 // number of steps whose log entries are written, published with a system-scope fence so
 // that the host may launch work on them while this runs.
-__device__ __forceinline__ void eph_emit(const PlanetConsts& pc, int nsteps, const EphRing& ring,
+__device__ __forceinline__ void eph_emit(const PlanetConsts& pc, double dt, int nsteps, const EphRing& ring,
                                          double* __restrict__ log, double* __restrict__ hist, int* progress) {
     const int np = pc.np;
     const int lane = threadIdx.x & 31;
@@ -340,18 +351,8 @@ __device__ __forceinline__ void eph_emit(const PlanetConsts& pc, int nsteps, con
 #pragma unroll
         for (int d = 0; d < 3; ++d) h0[d] = -warp_total0(own * r[d], lane, np);
         double* L = log + (size_t)e * S;
-        if (on) {
-            L[kRec * lane + 0] = r[0];
-            L[kRec * lane + 1] = r[1];
-            L[kRec * lane + 2] = r[2];
-            L[kRec * lane + 3] = 0.0;
-        }
-        if (lane == 0) {
-            L[kRec * np + 0] = h0[0];
-            L[kRec * np + 1] = h0[1];
-            L[kRec * np + 2] = h0[2];
-            L[kRec * np + 3] = 0.0;
-        }
+        if (on) store_rec(L + kRec * lane, r[0], r[1], r[2], r[0], r[1], r[2]);
+        if (lane == 0) store_rec(L + kRec * np, h0[0], h0[1], h0[2], dt * h0[0], dt * h0[1], dt * h0[2]);
         if (hist) {  // the same pointer on every lane: the warp takes this branch together
             double* Hs = hist + (size_t)e * 6 * np;
 #pragma unroll
@@ -381,7 +382,7 @@ __device__ __forceinline__ void eph_advance(const PlanetConsts& pc, double* jac,
         else
             eph_dynamics<1>(pc, jac, dt, nsteps, ring, status);
     } else {
-        eph_emit(pc, nsteps, ring, log, hist, progress);
+        eph_emit(pc, dt, nsteps, ring, log, hist, progress);
     }
 }
 
@@ -394,7 +395,7 @@ __global__ void __launch_bounds__(kEphThreads) eph_chunk_kernel(const PlanetCons
 
 // Many independent systems: block b advances system b.
 //   jac  : [n_sys][2][kMaxPlanets][3] Jacobi states (per-system stride 6 kMaxPlanets)
-//   log  : system b's log at log + log_off[b] (stride 4 (np_b + 1) doubles per step)
+//   log  : system b's log at log + log_off[b] (stride log_stride(np_b) doubles per step)
 //   dt   : [n_sys] steps
 __global__ void __launch_bounds__(kEphThreads) eph_batch_kernel(const PlanetConsts* __restrict__ pcs, double* jac,
                                                                   const double* __restrict__ dt, int nsteps,
@@ -409,7 +410,7 @@ __global__ void __launch_bounds__(kEphThreads) eph_batch_kernel(const PlanetCons
 //   pos : [n+1][np][3] heliocentric positions
 // ---------------------------------------------------------------------------
 __global__ void eph_external_kernel(const PlanetConsts* __restrict__ pcp, const double* __restrict__ pos, int64_t n1,
-                                    double* __restrict__ log) {
+                                    double dt, double* __restrict__ log) {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= n1) return;
     const int np = pcp->np;
@@ -422,15 +423,9 @@ __global__ void eph_external_kernel(const PlanetConsts* __restrict__ pcp, const 
         hx = fma(-s, x, hx);
         hy = fma(-s, y, hy);
         hz = fma(-s, z, hz);
-        log[k * S + kRec * j + 0] = x;
-        log[k * S + kRec * j + 1] = y;
-        log[k * S + kRec * j + 2] = z;
-        log[k * S + kRec * j + 3] = 0.0;
+        store_rec(log + k * S + kRec * j, x, y, z, x, y, z);
     }
-    log[k * S + kRec * np + 0] = hx;
-    log[k * S + kRec * np + 1] = hy;
-    log[k * S + kRec * np + 2] = hz;
-    log[k * S + kRec * np + 3] = 0.0;
+    store_rec(log + k * S + kRec * np, hx, hy, hz, dt * hx, dt * hy, dt * hz);
 }
 
 // host launchers ----------------------------------------------------------------
@@ -472,10 +467,11 @@ cudaError_t launch_eph_batch(const PlanetConsts* pcs, int n_sys, double* jac, co
     return cudaGetLastError();
 }
 
-cudaError_t launch_eph_external(const PlanetConsts* pc, const double* pos, int64_t n1, double* log, cudaStream_t s) {
+cudaError_t launch_eph_external(const PlanetConsts* pc, const double* pos, int64_t n1, double dt, double* log,
+                                cudaStream_t s) {
     const int bs = 128;
     const int64_t grid = (n1 + bs - 1) / bs;
-    eph_external_kernel<<<(unsigned)grid, bs, 0, s>>>(pc, pos, n1, log);
+    eph_external_kernel<<<(unsigned)grid, bs, 0, s>>>(pc, pos, n1, dt, log);
     return cudaGetLastError();
 }
 

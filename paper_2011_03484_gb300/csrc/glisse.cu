@@ -7,7 +7,7 @@
 //   alive       [cap] uint8 written by the particle kernel, reset after compaction
 //   per-id out  [N][6] state, [N] removal step, [N] reason
 //   planets     constants, Jacobi state [2][N_p][3]
-//   planet log  a ring of 3 chunk buffers, each [(C+1)][4 (N_p+1)] doubles of
+//   planet log  a ring of 3 chunk buffers, each [(C+1)][8 (N_p+1)] doubles of
 //               positions + h0, and [(C+1)][N_p][6] synchronised heliocentric
 //               states (for glisse_read_planets)
 //
@@ -40,7 +40,7 @@ cudaError_t launch_eph_setup(const double*, int, double, double, int, double, Pl
                              cudaStream_t);
 cudaError_t launch_eph_chunk(const PlanetConsts*, double*, double, int, double*, double*, int*, cudaStream_t,
                              int* progress = nullptr);
-cudaError_t launch_eph_external(const PlanetConsts*, const double*, int64_t, double*, cudaStream_t);
+cudaError_t launch_eph_external(const PlanetConsts*, const double*, int64_t, double, double*, cudaStream_t);
 cudaError_t launch_particle_chunk(int, const ChunkArgs&, const ParticleConsts&, cudaStream_t, const TaskArgs*, bool);
 cudaError_t launch_particle_chunk_paper(int, const ChunkArgs&, const ParticleConsts&, cudaStream_t);
 cudaError_t launch_compact(int64_t, const uint8_t*, const double*, const int32_t*, int64_t, double*, int32_t*,
@@ -92,7 +92,7 @@ constexpr int kPollGaveUp = 1;
 constexpr double kG = 4.0 * 3.14159265358979323846 * 3.14159265358979323846;
 }  // namespace
 
-// One chunk of planets on the device: log [(C+1)][4 (N_p+1)] (positions + h0)
+// One chunk of planets on the device: log [(C+1)][8 (N_p+1)] (positions + h0)
 // and history [(C+2)][N_p][6]: rows 0..C the synchronised heliocentric states,
 // row C+1 the planets' Jacobi state at the chunk's first step (what the planet
 // kernel started from; a checkpoint saves it so that resume recomputes the
@@ -1297,7 +1297,7 @@ extern "C" int glisse_set_ephemeris(glisse_ctx* c, const double* log, int64_t n_
         GL_ALLOC(d_pos, sizeof(double) * (size_t)(n_steps + 1) * 3 * c->np);
         cudaError_t e = cudaMemcpyAsync(d_pos, log, sizeof(double) * (size_t)(n_steps + 1) * 3 * c->np,
                                         cudaMemcpyHostToDevice, c->s);
-        if (e == cudaSuccess) e = launch_eph_external(c->d_pc, d_pos, n_steps + 1, c->d_ext_log, c->s);
+        if (e == cudaSuccess) e = launch_eph_external(c->d_pc, d_pos, n_steps + 1, c->dt, c->d_ext_log, c->s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->s);
         cudaFree(d_pos);
         if (e != cudaSuccess) return GLISSE_E_CUDA;

@@ -34,11 +34,14 @@ inline cudaError_t residency_cap_smem(const void* kernel, int64_t per_sm, int ma
 
 constexpr int kMaxPlanets = GLISSE_MAX_PLANETS;
 
-// One record per body per step in the planet log: heliocentric x, y, z and a pad.
-// A log step holds N_p planet records followed by the record of the common
-// term h0 = -sum_j G m_j r_j / |r_j|^3 (section 2.2).  32-byte records let a
-// warp fetch a whole record with two 16-byte broadcast loads.
-constexpr int kRec = 4;
+// One record per body per step in the planet log: x, y, z and a pad as doubles,
+// then the same three as float pairs (split_math.cuh): xh, yh, zh, xl, yl, zl and a
+// pad of two floats.  A log step holds N_p planet records (heliocentric positions)
+// followed by the record of the common term h0 = -sum_j G m_j r_j / |r_j|^3
+// (section 2.2), whose pairs hold dt h0.  The particle kernels fetch a record's
+// pairs with a 16-byte and an 8-byte broadcast load.
+constexpr int kRec = 8;
+constexpr int kRecSplit = 4;  // the pairs' offset in a record, in doubles
 __host__ __device__ constexpr int log_stride(int np) { return kRec * (np + 1); }
 // The ephemeris kernel of a context's first chunk publishes its step count this often.
 constexpr int kProgressEvery = 16;

@@ -32,6 +32,7 @@
 #include <algorithm>
 #include "glisse_internal.h"
 #include "kepler.cuh"
+#include "split_step.cuh"
 
 namespace glisse {
 
@@ -41,7 +42,7 @@ constexpr int kParticleBlock = 128;
 // that spills past one wave leaves a tail in which a lone warp per SM
 // partition cannot keep the FP64 pipe busy.
 #ifndef GLISSE_PARTICLE_MIN_BLOCKS
-#define GLISSE_PARTICLE_MIN_BLOCKS 8
+#define GLISSE_PARTICLE_MIN_BLOCKS 4
 #endif
 
 // drift used by the particle map: the converged fast solver (default) or the
@@ -49,7 +50,7 @@ constexpr int kParticleBlock = 128;
 constexpr int kDriftConverge = 0;
 constexpr int kDriftPaper = 1;
 
-// Read-only broadcast load of one 32-byte log record.
+// Read-only broadcast loads of one log record: its doubles, and its pairs.
 __device__ __forceinline__ void load_rec(const double* __restrict__ p, double& x, double& y, double& z) {
     const double2 a = __ldg(reinterpret_cast<const double2*>(p));
     x = a.x;
@@ -57,81 +58,118 @@ __device__ __forceinline__ void load_rec(const double* __restrict__ p, double& x
     z = __ldg(p + 2);
 }
 
-// Kick with the log step L by tau (tgm[j] = tau G m_j), and the encounter test.
-// Returns the lowest 1-based planet index whose test fires, or 0.
+__device__ __forceinline__ void load_rec_split(const double* __restrict__ p, F2 (&v)[3]) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p + kRecSplit));
+    const float2 b = __ldg(reinterpret_cast<const float2*>(p + kRecSplit + 2));
+    v[0] = F2{a.x, a.w};
+    v[1] = F2{a.y, b.x};
+    v[2] = F2{a.z, b.y};
+}
+
+// The terms that kick_sum leaves to FP64 (bit j of `near`: planet j, bit NP: h0), for
+// one lane: added to K, with the encounter test.  Returns the lowest 1-based
+// planet index whose test fires, or 0.
 template <int NP>
-__device__ __forceinline__ int kick_test(double x, double y, double z, double& vx, double& vy, double& vz,
-                                         const double* __restrict__ L, double tau, const double (&tgm)[kMaxPlanets],
-                                         const double (&rc2)[kMaxPlanets]) {
-    double hx, hy, hz;
-    load_rec(L + kRec * NP, hx, hy, hz);
-    vx = fma(tau, hx, vx);
-    vy = fma(tau, hy, vy);
-    vz = fma(tau, hz, vz);
+__device__ __noinline__ int kick_near(unsigned near, double x, double y, double z, const double* __restrict__ L,
+                                      const ParticleConsts& pc, double (&K)[3]) {
     int hit = 0;
-#pragma unroll
+    if ((near >> NP) & 1u) {
+        double hx, hy, hz;
+        load_rec(L + kRec * NP, hx, hy, hz);
+        K[0] = fma(pc.dt, hx, K[0]);
+        K[1] = fma(pc.dt, hy, K[1]);
+        K[2] = fma(pc.dt, hz, K[2]);
+    }
     for (int j = NP - 1; j >= 0; --j) {
+        if (!((near >> j) & 1u)) continue;
         double px, py, pz;
         load_rec(L + kRec * j, px, py, pz);
         const double dx = x - px, dy = y - py, dz = z - pz;
         const double d2 = fma(dx, dx, fma(dy, dy, dz * dz));
-        hit = lt_nonneg(d2, rc2[j]) ? (j + 1) : hit;
-        const double s = k_rcube(d2, tgm[j]);
-        vx = fma(-s, dx, vx);
-        vy = fma(-s, dy, vy);
-        vz = fma(-s, dz, vz);
+        hit = lt_nonneg(d2, pc.rc2[j]) ? (j + 1) : hit;
+        const double s = k_rcube(d2, pc.tgm_full[j]);
+        K[0] = fma(-s, dx, K[0]);
+        K[1] = fma(-s, dy, K[1]);
+        K[2] = fma(-s, dz, K[2]);
     }
     return hit;
 }
 
-// kick_test with the planets split over a lane pair (two lanes per particle,
-// both holding the same state): lane parity p takes planets p, p + 2, ...,
-// each lane sums its partial kick, and the pair adds the two partial sums (the
-// same sum on both lanes: addition commutes) and takes the lower encounter
-// index.  The h0 term is applied by both lanes as in kick_test.
-template <int NP>
-__device__ __forceinline__ int kick_test_pair(double x, double y, double z, double& vx, double& vy, double& vz,
-                                              const double* __restrict__ L, double tau,
-                                              const double (&tgm)[kMaxPlanets], const double (&rc2)[kMaxPlanets]) {
-    const int parity = threadIdx.x & 1;
-    double hx, hy, hz;
-    load_rec(L + kRec * NP, hx, hy, hz);
-    vx = fma(tau, hx, vx);
-    vy = fma(tau, hy, vy);
-    vz = fma(tau, hz, vz);
-    double ax = 0.0, ay = 0.0, az = 0.0;
-    int hit = 0;
+// The kick of a full step, K = dt a(r) at log step L (a half kick is exactly half
+// of it), and the encounter test: h0 and the planets in pairs (kick_split), in
+// FP64 the planets a lane is near to, and the whole sum where it exceeds 2^-7 |v|
+// (far out, where h0 outweighs the star: a pair's 46 bits of K would show in v).
+// X: the position split; sp.v2 is negative where the position is out of the
+// floats' range (then all is FP64).  Returns the lowest 1-based planet index whose
+// test fires, or 0.  All lanes of a warp call it together.
+// TPP = 2: a lane pair (both lanes holding the same particle) splits the planets:
+// lane parity p takes planets p, p + 2, ..., the partial sums are added (the
+// same bits on both lanes: two_sum and addition commute) and the lower index wins.
+template <int NP, int TPP>
+__device__ __forceinline__ int kick_sum(double x, double y, double z, const F2 (&X)[3], const Speed& sp, bool act,
+                                        const double* __restrict__ L, const ParticleConsts& pc, const SplitConsts& sc,
+                                        double (&K)[3]) {
+    const int parity = TPP == 2 ? (int)(threadIdx.x & 1) : 0;
+    const float lim2 = kSplitNear2 * sp.rate2;
+    F2 acc[3];
+    load_rec_split(L + kRec * NP, acc);
+    if (TPP == 2 && parity == 1) acc[0] = acc[1] = acc[2] = F2{0.0f, 0.0f};
+    unsigned near = 0, mine = parity == 0 ? 1u << NP : 0u;
 #pragma unroll
-    for (int jj = (NP + 1) / 2 - 1; jj >= 0; --jj) {
-        const int j = 2 * jj + parity;
+    for (int jj = (NP + TPP - 1) / TPP - 1; jj >= 0; --jj) {
+        const int j = TPP * jj + parity;
         if (j < NP) {
-            double px, py, pz;
-            load_rec(L + kRec * j, px, py, pz);
-            const double dx = x - px, dy = y - py, dz = z - pz;
-            const double d2 = fma(dx, dx, fma(dy, dy, dz * dz));
-            hit = lt_nonneg(d2, rc2[j]) ? (j + 1) : hit;
-            const double s = k_rcube(d2, tgm[j]);
-            ax = fma(-s, dx, ax);
-            ay = fma(-s, dy, ay);
-            az = fma(-s, dz, az);
+            F2 P[3];
+            load_rec_split(L + kRec * j, P);
+            if (!kick_split(X, P, sc.tg[j], sc.rc2[j], lim2, acc)) near |= 1u << j;
+            mine |= 1u << j;
         }
     }
-    vx += ax + __shfl_xor_sync(kFullMask, ax, 1);
-    vy += ay + __shfl_xor_sync(kFullMask, ay, 1);
-    vz += az + __shfl_xor_sync(kFullMask, az, 1);
-    const int other = __shfl_xor_sync(kFullMask, hit, 1);
-    return (hit != 0 && other != 0) ? min(hit, other) : (hit | other);
+    if constexpr (TPP == 2) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float oh = __shfl_xor_sync(kFullMask, acc[c].h, 1), ol = __shfl_xor_sync(kFullMask, acc[c].l, 1);
+            float e;
+            two_sum(acc[c].h, oh, acc[c].h, e);
+            acc[c].l = __fadd_rn(e, __fadd_rn(acc[c].l, ol));
+        }
+    }
+    const float k2 = fmaf(acc[0].h, acc[0].h, fmaf(acc[1].h, acc[1].h, acc[2].h * acc[2].h));
+    const bool small = k2 <= kSplitKick2 * sp.v2;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) K[c] = f2_double(f2_norm(acc[c].h, acc[c].l));
+    int hit = 0;
+    if (__any_sync(kFullMask, act && (near != 0u || !small))) {
+        if (!small) {
+            near = mine;
+            K[0] = K[1] = K[2] = 0.0;
+        }
+        if (!act) near = 0;
+        if constexpr (TPP == 2) {
+            double N[3] = {0.0, 0.0, 0.0};
+            hit = kick_near<NP>(near, x, y, z, L, pc, N);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) K[c] += N[c] + __shfl_xor_sync(kFullMask, N[c], 1);
+            const int other = __shfl_xor_sync(kFullMask, hit, 1);
+            hit = (hit != 0 && other != 0) ? min(hit, other) : (hit | other);
+        } else {
+            if (near) hit = kick_near<NP>(near, x, y, z, L, pc, K);
+        }
+    }
+    return hit;
 }
 
-// The kick of a particle held by TPP lanes (1, or 2: kick_test_pair).
-template <int NP, int TPP>
-__device__ __forceinline__ int kick_lanes(double x, double y, double z, double& vx, double& vy, double& vz,
-                                          const double* __restrict__ L, double tau, const double (&tgm)[kMaxPlanets],
-                                          const double (&rc2)[kMaxPlanets]) {
-    if constexpr (TPP == 2)
-        return kick_test_pair<NP>(x, y, z, vx, vy, vz, L, tau, tgm, rc2);
-    else
-        return kick_test<NP>(x, y, z, vx, vy, vz, L, tau, tgm, rc2);
+// The FP64 drift (kepler.cuh) of the lanes that drift_split leaves (part): the fast
+// path, then the general solver for lanes outside its domain.  Returns false for a
+// lane whose solve failed.  All lanes of a warp call it together.
+static __device__ __noinline__ bool drift_fp64(const ParticleConsts& pc, bool part, double (&s)[6]) {
+    double r0, mur0;
+    radius_of(s[0], s[1], s[2], r0, mur0);
+    mur0 *= pc.mu;
+    const bool done = drift_fast(pc.mu, d2f_bits(pc.mu), pc.dt, d2f_bits(pc.dt), part, r0, mur0, s[0], s[1], s[2],
+                                 s[3], s[4], s[5]);
+    if (part && !done) return drift_general(pc.mu, pc.dt, s[0], s[1], s[2], s[3], s[4], s[5]);
+    return true;
 }
 
 // Removal test without a kick (used at t_0).
@@ -173,12 +211,11 @@ struct PublishTo {
 // closing half kick), straight to memory so that nothing stays live in
 // registers across the steps.
 template <int NP, int MODE = kDriftConverge, int TPP = 1, bool PUBLISH = false>
-__device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const double* __restrict__ L, int64_t step0,
-                                             int nsteps, bool test_first, double& x, double& y, double& z, double& vx,
-                                             double& vy, double& vz, bool& act, int& reason, int64_t& rstep,
-                                             bool open_in = false, bool close_out = true, PublishTo pub = {}) {
-    const float muf = d2f_bits(pc.mu), dtf = d2f_bits(pc.dt);
-    const bool has_rmax = __double_as_longlong(pc.rmax) != 0;
+__device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const SplitConsts& sc,
+                                             const double* __restrict__ L, int64_t step0, int nsteps, bool test_first,
+                                             double& x, double& y, double& z, double& vx, double& vy, double& vz,
+                                             bool& act, int& reason, int64_t& rstep, bool open_in = false,
+                                             bool close_out = true, PublishTo pub = {}) {
     const int S = log_stride(NP);
 
     if (test_first) {
@@ -189,79 +226,92 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const dou
             rstep = step0;
         }
     }
+    F2 X[3] = {f2_split(x), f2_split(y), f2_split(z)};
+    double r2 = fma(x, x, fma(y, y, z * z));
     if (!open_in) {
-        if constexpr (TPP == 2) {
-            // the pair kick shuffles across the warp: every lane runs it, active lanes keep it
-            double nvx = vx, nvy = vy, nvz = vz;
-            kick_test_pair<NP>(x, y, z, nvx, nvy, nvz, L, pc.half_dt, pc.tgm_half, pc.rc2);
-            if (act) {
-                vx = nvx;
-                vy = nvy;
-                vz = nvz;
-            }
-        } else if (act) {
-            kick_test<NP>(x, y, z, vx, vy, vz, L, pc.half_dt, pc.tgm_half, pc.rc2);
+        double K[3];
+        kick_sum<NP, TPP>(x, y, z, X, float_speed(r2, vx, vy, vz), act, L, pc, sc, K);
+        if (act) {
+            vx = fma(0.5, K[0], vx);
+            vy = fma(0.5, K[1], vy);
+            vz = fma(0.5, K[2], vz);
         }
     }
-    double r0, mur0;
-    radius_of(x, y, z, r0, mur0);
-    mur0 *= pc.mu;
 
     for (int k = 0; k < nsteps; ++k) {
         if (!__any_sync(kFullMask, act)) break;
         const double* __restrict__ Ln = L + (size_t)(k + 1) * S;
-        const double sx = x, sy = y, sz = z, svx = vx, svy = vy, svz = vz;
-        const double sr0 = r0, smur0 = mur0;
+        double n[6];
         bool failed = false;
+        Speed sp;
         if constexpr (MODE == kDriftConverge) {
-            const bool done = drift_fast(pc.mu, muf, pc.dt, dtf, act, r0, mur0, x, y, z, vx, vy, vz);
-            if (act && !done) {
-                failed = !drift_general(pc.mu, pc.dt, x, y, z, vx, vy, vz);
-                radius_of(x, y, z, r0, mur0);
-                mur0 *= pc.mu;
+            const F2 V[3] = {f2_split(vx), f2_split(vy), f2_split(vz)};
+            DriftFactors f;
+            const bool fast = drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp) && act;
+            n[0] = fma(f.fm1, x, fma(f.g, vx, x));
+            n[1] = fma(f.fm1, y, fma(f.g, vy, y));
+            n[2] = fma(f.fm1, z, fma(f.g, vz, z));
+            n[3] = fma(f.fd, x, fma(f.gdm1, vx, vx));
+            n[4] = fma(f.fd, y, fma(f.gdm1, vy, vy));
+            n[5] = fma(f.fd, z, fma(f.gdm1, vz, vz));
+            const bool slow = act && !fast;
+            if (__any_sync(kFullMask, slow)) {
+                double s[6] = {x, y, z, vx, vy, vz};
+                const bool done = drift_fp64(pc, slow, s);
+                if (slow) {
+                    failed = !done;
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) n[c] = s[c];
+                }
             }
         } else {
-            if (act) {
-                failed = drift_paper(pc.mu, pc.dt, pc.kepler_iters, pc.kepler_tol, x, y, z, vx, vy, vz) != 0;
-                radius_of(x, y, z, r0, mur0);
-            }
+            sp = float_speed(r2, vx, vy, vz);
+            n[0] = x;
+            n[1] = y;
+            n[2] = z;
+            n[3] = vx;
+            n[4] = vy;
+            n[5] = vz;
+            if (act)
+                failed = drift_paper(pc.mu, pc.dt, pc.kepler_iters, pc.kepler_tol, n[0], n[1], n[2], n[3], n[4],
+                                     n[5]) != 0;
         }
-        const bool bad = nonfinite_bits(x) || nonfinite_bits(y) || nonfinite_bits(z) || nonfinite_bits(vx) ||
-                         nonfinite_bits(vy) || nonfinite_bits(vz);
+        const bool bad = nonfinite_bits(n[0]) || nonfinite_bits(n[1]) || nonfinite_bits(n[2]) ||
+                         nonfinite_bits(n[3]) || nonfinite_bits(n[4]) || nonfinite_bits(n[5]);
         if (act && (failed || bad)) {
-            x = sx;
-            y = sy;
-            z = sz;
-            vx = svx;
-            vy = svy;
-            vz = svz;
-            r0 = sr0;
-            mur0 = smur0;
+            // the state stays what it was before the drift
             act = false;
             reason = failed ? GLISSE_REMOVED_KEPLER : GLISSE_REMOVED_NONFINITE;
             rstep = step0 + k + 1;
         }
-        // escape: |r| > r_max, with |r| from the drift (integer compare of positive doubles)
-        int hit = (has_rmax && lt_nonneg(pc.rmax, r0)) ? GLISSE_REMOVED_ESCAPE : 0;
-        const bool last = close_out && (k + 1 == nsteps);
-        double nvx = vx, nvy = vy, nvz = vz;
-        int enc;
-        if (last)
-            enc = kick_lanes<NP, TPP>(x, y, z, nvx, nvy, nvz, Ln, pc.half_dt, pc.tgm_half, pc.rc2);
-        else
-            enc = kick_lanes<NP, TPP>(x, y, z, nvx, nvy, nvz, Ln, pc.dt, pc.tgm_full, pc.rc2);
+        if (act) {
+            x = n[0];
+            y = n[1];
+            z = n[2];
+            vx = n[3];
+            vy = n[4];
+            vz = n[5];
+        }
+        X[0] = f2_split(x);
+        X[1] = f2_split(y);
+        X[2] = f2_split(z);
+        r2 = fma(x, x, fma(y, y, z * z));
+        // escape: |r|^2 > r_max^2 (integer compare of non-negative doubles)
+        int hit = (__double_as_longlong(pc.rmax2) != 0 && lt_nonneg(pc.rmax2, r2)) ? GLISSE_REMOVED_ESCAPE : 0;
+        if (!in_float_range(r2)) sp.v2 = -1.0f;
+        double K[3];
+        const int enc = kick_sum<NP, TPP>(x, y, z, X, sp, act, Ln, pc, sc, K);
         hit = enc ? enc : hit;
+        const bool last = k + 1 == nsteps;
         if constexpr (PUBLISH) {
-            if (pub.out && !close_out && k + 1 == nsteps && act && hit == 0) {
-                double hx = vx, hy = vy, hz = vz;
-                kick_test<NP>(x, y, z, hx, hy, hz, Ln, pc.half_dt, pc.tgm_half, pc.rc2);
+            if (pub.out && !close_out && last && act && hit == 0) {
                 double* o = pub.out + 6 * (int64_t)pub.id[pub.slot];
                 o[0] = x;
                 o[1] = y;
                 o[2] = z;
-                o[3] = hx;
-                o[4] = hy;
-                o[5] = hz;
+                o[3] = fma(0.5, K[0], vx);
+                o[4] = fma(0.5, K[1], vy);
+                o[5] = fma(0.5, K[2], vz);
             }
         }
         if (act) {
@@ -269,10 +319,14 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const dou
                 act = false;
                 reason = hit;
                 rstep = step0 + k + 1;
+            } else if (close_out && last) {
+                vx = fma(0.5, K[0], vx);
+                vy = fma(0.5, K[1], vy);
+                vz = fma(0.5, K[2], vz);
             } else {
-                vx = nvx;
-                vy = nvy;
-                vz = nvz;
+                vx += K[0];
+                vy += K[1];
+                vz += K[2];
             }
         }
     }
@@ -295,7 +349,7 @@ __device__ __forceinline__ void store_removed(int64_t pid, double x, double y, d
 
 template <int NP, int MODE>
 __global__ void __launch_bounds__(kParticleBlock, GLISSE_PARTICLE_MIN_BLOCKS)
-    particle_chunk_kernel(const ChunkArgs a, const ParticleConsts pc) {
+    particle_chunk_kernel(const ChunkArgs a, const ParticleConsts pc, const SplitConsts sc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool in = i < a.n;
     const int64_t ld = a.ld;
@@ -320,7 +374,7 @@ __global__ void __launch_bounds__(kParticleBlock, GLISSE_PARTICLE_MIN_BLOCKS)
     const bool started = act;
     int reason = 0;
     int64_t rstep = -1;
-    advance_lane<NP, MODE, 1, true>(pc, a.log, a.step0, a.nsteps, a.test_first != 0, x, y, z, vx, vy, vz, act,
+    advance_lane<NP, MODE, 1, true>(pc, sc, a.log, a.step0, a.nsteps, a.test_first != 0, x, y, z, vx, vy, vz, act,
                                     reason, rstep, a.open_in != 0, a.close_out != 0, PublishTo{a.id, a.out_state, i});
     if (a.steps_done) {
         // steps this particle actually advanced in the segment (exact work count)
@@ -385,7 +439,7 @@ constexpr int kTaskMaxBlocks = 4;
 
 template <int NP>
 __global__ void __launch_bounds__(kParticleBlock, kTaskMaxBlocks)
-    particle_tasks_kernel(const ChunkArgs a, const ParticleConsts pc, const TaskArgs ta) {
+    particle_tasks_kernel(const ChunkArgs a, const ParticleConsts pc, const SplitConsts sc, const TaskArgs ta) {
     const int lane = threadIdx.x & 31;
     const int64_t ld = a.ld;
     const int S = log_stride(NP);
@@ -433,7 +487,7 @@ __global__ void __launch_bounds__(kParticleBlock, kTaskMaxBlocks)
         const int k0 = s * ta.sub_steps;
         const int m = min(ta.sub_steps, a.nsteps - k0);
         const bool last = s + 1 == n_sub;
-        advance_lane<NP, kDriftConverge, 1, true>(pc, a.log + (size_t)k0 * S, a.step0 + k0, m,
+        advance_lane<NP, kDriftConverge, 1, true>(pc, sc, a.log + (size_t)k0 * S, a.step0 + k0, m,
                                                   a.test_first != 0 && s == 0, x, y, z, vx, vy, vz, act, reason,
                                                   rstep, s > 0 || a.open_in != 0, last ? a.close_out != 0 : false,
                                                   PublishTo{a.id, last ? a.out_state : nullptr, i});
@@ -499,6 +553,9 @@ template <int MODE>
 cudaError_t launch_particle_chunk_mode(int np, const ChunkArgs& a, const ParticleConsts& pc, cudaStream_t s,
                                        const TaskArgs* tb = nullptr, bool force_tasks = false) {
     if (a.n <= 0) return cudaSuccess;
+    SplitConsts sc{};
+    split_step_consts(pc, sc);
+    for (int j = 0; j < kMaxPlanets; ++j) split_planet(pc, j, sc);
     if constexpr (MODE == kDriftConverge) {
         int dev = 0, nsm = 0;
         cudaError_t e = cudaGetDevice(&dev);
@@ -521,7 +578,7 @@ cudaError_t launch_particle_chunk_mode(int np, const ChunkArgs& a, const Particl
     case N:                                                                                              \
         e = particle_smem_cap(reinterpret_cast<const void*>(particle_tasks_kernel<N>), grid, &smem);     \
         if (e != cudaSuccess) return e;                                                                  \
-        particle_tasks_kernel<N><<<(unsigned)grid, kParticleBlock, smem, s>>>(a, pc, b);                 \
+        particle_tasks_kernel<N><<<(unsigned)grid, kParticleBlock, smem, s>>>(a, pc, sc, b);                 \
         break;
                 GLISSE_TCASE(0)
                 GLISSE_TCASE(1)
@@ -546,7 +603,7 @@ cudaError_t launch_particle_chunk_mode(int np, const ChunkArgs& a, const Particl
     case N:                                                                                               \
         e = particle_smem_cap(reinterpret_cast<const void*>(particle_chunk_kernel<N, MODE>), grid, &smem); \
         if (e != cudaSuccess) return e;                                                                   \
-        particle_chunk_kernel<N, MODE><<<(unsigned)grid, kParticleBlock, smem, s>>>(a, pc);              \
+        particle_chunk_kernel<N, MODE><<<(unsigned)grid, kParticleBlock, smem, s>>>(a, pc, sc);              \
         break;
         GLISSE_CASE(0)
         GLISSE_CASE(1)

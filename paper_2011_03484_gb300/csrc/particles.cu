@@ -13,8 +13,9 @@ namespace glisse {
 // holds particle start + k (half of the task's 32 particles per call; `half`
 // picks which), and only its even lane writes results and counts.
 template <int NP, int TPP>
-__device__ __forceinline__ void batch_task(const BatchArgs& a, const ParticleConsts& pc, int s, int64_t start,
-                                           int cnt, int lane, int64_t step0, bool test_first, int half = 0) {
+__device__ __forceinline__ void batch_task(const BatchArgs& a, const ParticleConsts& pc, const SplitConsts& sc,
+                                           int s, int64_t start, int cnt, int lane, int64_t step0, bool test_first,
+                                           int half = 0) {
     const int slot = TPP == 2 ? 16 * half + (lane >> 1) : lane;
     const bool owner = TPP == 1 || (lane & 1) == 0;
     const int64_t i = start + slot;
@@ -33,7 +34,7 @@ __device__ __forceinline__ void batch_task(const BatchArgs& a, const ParticleCon
     const bool started = act;
     int reason = 0;
     int64_t rstep = -1;
-    advance_lane<NP, kDriftConverge, TPP>(pc, a.log + a.log_off[s], step0, a.nsteps, test_first, x, y, z, vx, vy, vz,
+    advance_lane<NP, kDriftConverge, TPP>(pc, sc, a.log + a.log_off[s], step0, a.nsteps, test_first, x, y, z, vx, vy, vz,
                                           act, reason, rstep);
     const unsigned live = __reduce_add_sync(kFullMask, (act && owner) ? 1u : 0u);
     if (lane == 0 && live) atomicAdd(reinterpret_cast<unsigned long long*>(a.cnt_new + s), (unsigned long long)live);
@@ -61,6 +62,7 @@ constexpr int kBatchMaxWarps = 8;  // largest block of the batched kernel: 256 t
 template <int TPP>
 __global__ void __launch_bounds__(32 * kBatchMaxWarps) batch_particle_kernel(const BatchArgs a) {
     __shared__ ParticleConsts s_pc[kBatchMaxWarps];
+    __shared__ SplitConsts s_sc[kBatchMaxWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntask = *a.n_tasks;
     const int64_t step0 = a.clock->step;
@@ -79,11 +81,15 @@ __global__ void __launch_bounds__(32 * kBatchMaxWarps) batch_particle_kernel(con
         double* dst = reinterpret_cast<double*>(&s_pc[warp]);
         for (int w = lane; w < kWords; w += 32) dst[w] = src[w];
         __syncwarp();
+        if (lane < kMaxPlanets) split_planet(s_pc[warp], lane, s_sc[warp]);
+        if (lane == kMaxPlanets) split_step_consts(s_pc[warp], s_sc[warp]);
+        __syncwarp();
         const ParticleConsts& pc = s_pc[warp];
+        const SplitConsts& sc = s_sc[warp];
         switch (a.np_of[s]) {
 #define GLISSE_BCASE(N)                                                          \
     case N:                                                                      \
-        for (int h = 0; h < TPP; ++h) batch_task<N, TPP>(a, pc, s, start, cnt, lane, step0, test_first, h); \
+        for (int h = 0; h < TPP; ++h) batch_task<N, TPP>(a, pc, sc, s, start, cnt, lane, step0, test_first, h); \
         break;
             GLISSE_BCASE(0)
             GLISSE_BCASE(1)
@@ -151,7 +157,7 @@ cudaError_t particle_wait_selftest(int polls, char* scratch, int* status, cudaSt
     const unsigned long long first = kGroups;
     cudaError_t e = cudaMemcpyAsync(ta.task_counter, &first, sizeof(first), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
-    particle_tasks_kernel<0><<<4, kParticleBlock, 0, s>>>(a, ParticleConsts{}, ta);
+    particle_tasks_kernel<0><<<4, kParticleBlock, 0, s>>>(a, ParticleConsts{}, SplitConsts{}, ta);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     return e;

@@ -1,0 +1,123 @@
+// split_math.cuh -- numbers held as an unevaluated sum of two floats.
+//
+// A GB300 SM partition issues an FP64 instruction of a warp every 64 cycles and
+// an FP32 one every cycle, so a product of two pairs (4 instructions) or a sum
+// (8) costs an eighth of the FP64 one it stands for.  A pair carries 46 to 48
+// significant bits.  It is used where its value enters a double as a small
+// correction (a kick against the velocity, f - 1 against 1), so that its error
+// lies below the rounding of that double; the sums themselves stay in FP64.
+//
+// Error-free transforms: Knuth's two-sum, Dekker's fast two-sum and the product
+// with its fused remainder.  The __f*_rn intrinsics keep the compiler from
+// contracting them.
+#pragma once
+#include "device_math.cuh"
+
+namespace glisse {
+
+struct F2 {
+    float h, l;
+};
+
+__device__ __forceinline__ float rsqrt_f32(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float rcp_f32(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// a + b = s + e exactly (6 instructions).
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// The same for |a| >= |b| (3 instructions).
+__device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    e = __fsub_rn(b, __fsub_rn(s, a));
+}
+
+__device__ __forceinline__ F2 f2_norm(float h, float l) {
+    F2 r;
+    fast_two_sum(h, l, r.h, r.l);
+    return r;
+}
+
+// Product; the low part may reach 2^-22 of the high one (not renormalised).
+__device__ __forceinline__ F2 f2_mul(const F2& a, const F2& b) {
+    F2 r;
+    r.h = __fmul_rn(a.h, b.h);
+    r.l = __fmaf_rn(a.h, b.h, -r.h);
+    r.l = __fmaf_rn(a.h, b.l, r.l);
+    r.l = __fmaf_rn(a.l, b.h, r.l);
+    return r;
+}
+
+__device__ __forceinline__ F2 f2_sub(const F2& a, const F2& b) {
+    F2 r;
+    float e;
+    two_sum(a.h, -b.h, r.h, e);
+    r.l = __fadd_rn(e, __fsub_rn(a.l, b.l));
+    return r;
+}
+
+// Quotient a / b with rb ~ 1 / b.h (2^-22).
+__device__ __forceinline__ F2 f2_div(const F2& a, const F2& b, float rb) {
+    F2 q;
+    q.h = __fmul_rn(a.h, rb);
+    float e = __fmaf_rn(-q.h, b.h, a.h);
+    e = __fadd_rn(__fmaf_rn(-q.h, b.l, e), a.l);
+    q.l = __fmul_rn(e, rb);
+    return q;
+}
+
+// (a.x b.x + a.y b.y) + a.z b.z from split vectors.
+__device__ __forceinline__ F2 f2_dot(const F2 (&a)[3], const F2 (&b)[3]) {
+    const F2 p = f2_mul(a[0], b[0]), q = f2_mul(a[1], b[1]), r = f2_mul(a[2], b[2]);
+    F2 s;
+    float e, f;
+    two_sum(p.h, q.h, s.h, e);
+    two_sum(s.h, r.h, s.h, f);
+    s.l = __fadd_rn(__fadd_rn(e, f), __fadd_rn(__fadd_rn(p.l, q.l), r.l));
+    return s;
+}
+
+// A double as a pair, by integer operations and one int-to-float conversion
+// (an F2F conversion occupies the FP64 pipe): the leading 24 bits, and the other
+// 29 rounded to 24.  |x| below 2^-74 is read as 2^-74 (1 + ...): far below
+// anything it is added to.  |x| must be below 2^127.
+__device__ __forceinline__ F2 f2_split(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned a = max(hi & 0x7FFFFFFFu, (unsigned)(1023 - 74) << 20);
+    const unsigned b = (__funnelshift_l(lo, a, 3) + 0x40000000u) | (hi & 0x80000000u);
+    F2 r;
+    r.h = __uint_as_float(b);
+    r.l = __fmul_rn((float)(int)(lo & 0x1FFFFFFFu), __uint_as_float((b & 0xFF800000u) - (52u << 23)));
+    return r;
+}
+
+// A normalised pair (|l| <= ulp(h)) as a double: h's bits moved to a double,
+// then l added to the significand as an integer in units of 2^-46 of h's binade
+// (l beyond them is dropped: below 2^-47 of the value).  Below a power of two
+// the significand's unit is half as large, so a negative l counts double there.
+// Pairs below 2^-80 lose their l.
+__device__ __forceinline__ double f2_double(const F2& v) {
+    const unsigned b = __float_as_uint(v.h);
+    const unsigned hw = ((unsigned)((int)b >> 3) & 0x8FFFFFFFu) + 0x38000000u;
+    const long long base = ((long long)hw << 32) | (b << 29);
+    // sign(h) 2^(46 - E): k = l / h's binade in units of 2^-46, toward h's sign
+    const float sc = __uint_as_float(((b ^ 0x7F800000u) & 0xFF800000u) + (45u << 23));
+    const float magic = 12582912.0f;  // 1.5 2^23
+    int k = (int)__float_as_uint(__fmaf_rn(v.l, sc, magic)) - 0x4B400000;
+    if (k < 0 && (b & 0x007FFFFFu) == 0u) k += k;
+    return __longlong_as_double(base + (long long)k * 64);
+}
+
+}  // namespace glisse

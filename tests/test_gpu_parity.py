@@ -568,3 +568,51 @@ def test_device_side_argument_errors(G):
     sim.advance(0)
     assert sim.status()[1] == 0
     sim.close()
+
+
+def _split_case(name, rng):
+    """(planets, particles, dt, steps, ulps) around the lines where the step's arithmetic changes:
+    the drift in float pairs up to (n dt)^2 = 2^-9, the kick in float pairs beyond a distance that
+    grows with the planet's mass, FP64 elsewhere."""
+    mu = G_
+    n = 333
+    pl = gi.planet_system(np.random.Generator(np.random.PCG64(7)))
+    ang = rng.uniform(0, 2 * np.pi, (3, n))
+    if name == "tiers":  # (n dt)^2 from 1e-7 to 0.3
+        a = np.exp(rng.uniform(np.log(3.0), np.log(600.0), n))
+        return pl[:0], gi.elements_to_cartesian(mu, a, rng.uniform(0, 0.9, n), rng.uniform(0, 3, n), *ang), 0.5, 4, 100
+    if name == "planar":  # z = vz = 0 exactly, some coordinates zero or denormal
+        p = gi.elements_to_cartesian(mu, rng.uniform(21, 28, n), rng.uniform(0, 0.1, n), np.zeros(n), *ang)
+        p[:, 2] = p[:, 5] = 0.0
+        p[0] = [25.0, 0.0, 0.0, 0.0, math.sqrt(mu / 25.0), 0.0]
+        p[1] = [0.0, -25.0, 1e-310, math.sqrt(mu / 25.0), -0.0, 1e-300]
+        return pl, p, 0.5, 4, 20
+    if name == "backward":
+        return pl, gi.elements_to_cartesian(mu, rng.uniform(21, 50, n), rng.uniform(0, 0.4, n),
+                                              0.1 * ang[0], *ang), -0.5, 4, 20
+    if name == "distant":  # far outside a float's square
+        a = np.exp(rng.uniform(np.log(1e3), np.log(1e25), n))
+        return pl, gi.elements_to_cartesian(mu, a, rng.uniform(0, 0.5, n), ang[0], *ang), 0.5, 2, 20
+    # "near": 0.3 to 8 Hill radii from each planet, moving with it (one step: a pass amplifies rounding)
+    j = rng.integers(0, 4, n)
+    rh = np.array(gi.PLANET_A) * (np.array(gi.PLANET_M) / 3.0) ** (1 / 3)
+    u = rng.normal(size=(n, 3))
+    u *= (rh[j] * np.exp(rng.uniform(np.log(0.3), np.log(8.0), n)) / np.linalg.norm(u, axis=1))[:, None]
+    p = pl[j, 1:].copy()
+    p[:, :3] += u
+    return pl, p, 0.01, 1, 20
+
+
+@pytest.mark.parametrize("name", ["tiers", "planar", "backward", "distant", "near"])
+def test_step_arithmetic_against_the_oracle(G, orc, name):
+    """A few steps against the oracle: each step rounds its sums a few times on either side, so a state
+    differs by some ulps of its norm per step (eccentric orbits near the pericentre: ten times that)."""
+    pl, pa, dt, steps, ulps = _split_case(name, np.random.Generator(np.random.PCG64(11)))
+    for mode in (G.GLISSE_LAUNCH_PLAIN, G.GLISSE_LAUNCH_TASKS):
+        sim = G.Simulation(1.0, pl, pa, dt, r_max=0.0, enc_value=0.0, launch_mode=mode)
+        sim.advance(steps)
+        got = sim.read()
+        sim.close()
+        ref = orc.run(1.0, pl, pa, dt, steps, r_max=0.0, k_hill=0.0)
+        assert got["alive"].all() and (ref["removal_step"] < 0).all()
+        assert parity.rel_err(got["state"], ref["state"]).max() < ulps * steps * 2.0**-53
