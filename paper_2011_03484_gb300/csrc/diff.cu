@@ -52,7 +52,7 @@ namespace glisse {
 cudaError_t launch_eph_setup(const double*, int, double, double, int, double, PlanetConsts*, double*, int*,
                              cudaStream_t);
 cudaError_t launch_eph_chunk(const PlanetConsts*, double*, double, int, double*, double*, int*, cudaStream_t,
-                             int* progress = nullptr);
+                             int* progress = nullptr, const int* stop = nullptr);
 
 constexpr int kMaxTangents = 6;
 constexpr int kScratchRows = 14;  // pre-drift state (6), post-drift position (3), s, tau, G_4, G_5, 1/R

@@ -39,7 +39,7 @@ namespace glisse {
 cudaError_t launch_eph_setup(const double*, int, double, double, int, double, PlanetConsts*, double*, int*,
                              cudaStream_t);
 cudaError_t launch_eph_chunk(const PlanetConsts*, double*, double, int, double*, double*, int*, cudaStream_t,
-                             int* progress = nullptr);
+                             int* progress = nullptr, const int* stop = nullptr);
 cudaError_t launch_eph_external(const PlanetConsts*, const double*, int64_t, double, double*, cudaStream_t);
 cudaError_t launch_particle_chunk(int, const ChunkArgs&, const ParticleConsts&, cudaStream_t, const TaskArgs*, bool);
 cudaError_t launch_particle_chunk_paper(int, const ChunkArgs&, const ParticleConsts&, cudaStream_t);
@@ -123,6 +123,7 @@ struct glisse_ctx {
     PlanetConsts* d_pc = nullptr;
     double* d_jac = nullptr;
     int* d_status = nullptr;
+    int* d_stop = nullptr;  // set to end the planet kernels in flight (destroy)
     int* h_status = nullptr;
     std::vector<Slot> ring;  // planet-log slots; chunk j lives in ring[j % ring.size()]
     cudaEvent_t ev_order = nullptr;
@@ -261,7 +262,12 @@ static bool alloc_slot(const glisse_ctx* c, Slot& sl) {
 
 static void ctx_free(glisse_ctx* c) {
     if (!c) return;
-    if (c->s) cudaStreamSynchronize(c->s);
+    if (c->s) {
+        // planet chunks running ahead of the particles are of no use any more: they look
+        // at the stop word every 16 steps
+        if (c->se && c->d_stop) cudaMemsetAsync(c->d_stop, 0xFF, sizeof(int), c->s);
+        cudaStreamSynchronize(c->s);
+    }
     if (c->se) cudaStreamSynchronize(c->se);
     for (Slot& sl : c->ring) free_slot(sl);
     for (cudaEvent_t e : {c->tp0, c->tp1, c->tc0, c->tc1, c->ev_order})
@@ -311,7 +317,8 @@ static int ensure_chunk(glisse_ctx* c, int64_t j) {
         if (c->np > 0)
             GL_CUDA(cudaMemcpyAsync(sl.hist + (size_t)(c->C + 1) * 6 * c->np, c->d_jac, sizeof(double) * 6 * c->np,
                                     cudaMemcpyDeviceToDevice, c->se));
-        GL_CUDA(launch_eph_chunk(c->d_pc, c->d_jac, c->dt, c->C, sl.log, sl.hist, c->d_status, c->se, prog));
+        GL_CUDA(launch_eph_chunk(c->d_pc, c->d_jac, c->dt, c->C, sl.log, sl.hist, c->d_status, c->se, prog,
+                                 c->d_stop));
         if (c->timing) {
             GL_CUDA(cudaEventRecord(sl.te1, c->se));
             sl.pending = true;
@@ -447,7 +454,7 @@ static int setup(glisse_ctx* c, const double* planets, const double* particles, 
             return o;
         };
         const size_t o_pc = take(sizeof(PlanetConsts)), o_jac = take(sizeof(double) * 6 * std::max(np, 1)),
-                     o_status = take(sizeof(int)), o_in = take(sizeof(double) * 7 * std::max(np, 1));
+                     o_status = take(sizeof(int)), o_stop = take(sizeof(int)), o_in = take(sizeof(double) * 7 * std::max(np, 1));
         size_t o_log[kRingMin], o_hist[kRingMin];
         for (size_t r = 0; r < kRingMin; ++r) {
             o_log[r] = take(sizeof(double) * (size_t)(c->C + 1) * S);
@@ -470,6 +477,7 @@ static int setup(glisse_ctx* c, const double* planets, const double* particles, 
         c->d_pc = reinterpret_cast<PlanetConsts*>(base + o_pc);
         c->d_jac = reinterpret_cast<double*>(base + o_jac);
         c->d_status = reinterpret_cast<int*>(base + o_status);
+        c->d_stop = reinterpret_cast<int*>(base + o_stop);
         d_in = reinterpret_cast<double*>(base + o_in);
         for (size_t r = 0; r < kRingMin; ++r) {
             c->ring[r].log = reinterpret_cast<double*>(base + o_log[r]);
@@ -496,6 +504,7 @@ static int setup(glisse_ctx* c, const double* planets, const double* particles, 
     for (Slot& sl : c->ring)
         if (!alloc_slot(c, sl)) return GLISSE_E_NOMEM;
     if (c->timing) GL_CUDA(cudaMemsetAsync(c->d_steps, 0, sizeof(unsigned long long), c->s));
+    GL_CUDA(cudaMemsetAsync(c->d_stop, 0, sizeof(int), c->s));  // before the stream's synchronisation below
 
     cudaError_t e = cudaSuccess;
     if (r) {

@@ -70,7 +70,7 @@ __device__ __forceinline__ void load_rec_split(const double* __restrict__ p, F2 
 // one lane: added to K, with the encounter test.  Returns the lowest 1-based
 // planet index whose test fires, or 0.
 template <int NP>
-__device__ __noinline__ int kick_near(unsigned near, double x, double y, double z, const double* __restrict__ L,
+__device__ __forceinline__ int kick_near(unsigned near, double x, double y, double z, const double* __restrict__ L,
                                       const ParticleConsts& pc, double (&K)[3]) {
     int hit = 0;
     if ((near >> NP) & 1u) {
@@ -80,6 +80,7 @@ __device__ __noinline__ int kick_near(unsigned near, double x, double y, double 
         K[1] = fma(pc.dt, hy, K[1]);
         K[2] = fma(pc.dt, hz, K[2]);
     }
+#pragma unroll 1
     for (int j = NP - 1; j >= 0; --j) {
         if (!((near >> j) & 1u)) continue;
         double px, py, pz;
@@ -152,8 +153,8 @@ __device__ __forceinline__ int kick_sum(double x, double y, double z, const F2 (
             for (int c = 0; c < 3; ++c) K[c] += N[c] + __shfl_xor_sync(kFullMask, N[c], 1);
             const int other = __shfl_xor_sync(kFullMask, hit, 1);
             hit = (hit != 0 && other != 0) ? min(hit, other) : (hit | other);
-        } else {
-            if (near) hit = kick_near<NP>(near, x, y, z, L, pc, K);
+        } else if (near) {
+            hit = kick_near<NP>(near, x, y, z, L, pc, K);
         }
     }
     return hit;

@@ -19,6 +19,12 @@ struct F2 {
     float h, l;
 };
 
+// x rounded to a pair (conversions: for constants)
+__host__ __device__ inline F2 f2_const(double x) {
+    const float h = (float)x;
+    return F2{h, (float)(x - (double)h)};
+}
+
 __device__ __forceinline__ float rsqrt_f32(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -60,6 +66,14 @@ __device__ __forceinline__ F2 f2_mul(const F2& a, const F2& b) {
     return r;
 }
 
+__device__ __forceinline__ F2 f2_add(const F2& a, const F2& b) {
+    F2 r;
+    float e;
+    two_sum(a.h, b.h, r.h, e);
+    r.l = __fadd_rn(e, __fadd_rn(a.l, b.l));
+    return r;
+}
+
 __device__ __forceinline__ F2 f2_sub(const F2& a, const F2& b) {
     F2 r;
     float e;
@@ -76,6 +90,54 @@ __device__ __forceinline__ F2 f2_div(const F2& a, const F2& b, float rb) {
     e = __fadd_rn(__fmaf_rn(-q.h, b.l, e), a.l);
     q.l = __fmul_rn(e, rb);
     return q;
+}
+
+// a - b c
+__device__ __forceinline__ F2 f2_fnma(const F2& b, const F2& c, const F2& a) { return f2_sub(a, f2_mul(b, c)); }
+
+// D^(-1/2) of a pair to 46 bits: y, y^2 = yy + yl exactly, e = 1 - D y^2 (below 2^-21).
+struct RsqrtF2 {
+    float y, yy, yl, e;
+};
+__device__ __forceinline__ RsqrtF2 f2_rsqrt(const F2& D) {
+    RsqrtF2 r;
+    r.y = rsqrt_f32(D.h);
+    r.yy = __fmul_rn(r.y, r.y);
+    r.yl = __fmaf_rn(r.y, r.y, -r.yy);
+    r.e = __fmaf_rn(-D.h, r.yy, 1.0f);
+    r.e = __fmaf_rn(-D.h, r.yl, r.e);
+    r.e = __fmaf_rn(-D.l, r.yy, r.e);
+    return r;
+}
+
+// k D^(-3/2) = k y^3 (1 - e)^(-3/2), k D^(-1) = k y^2 / (1 - e)
+__device__ __forceinline__ F2 f2_k_rcube(const RsqrtF2& r, const F2& k) {
+    const float y3 = __fmul_rn(r.y, r.yy);
+    const float y3l = __fmaf_rn(r.y, r.yl, __fmaf_rn(r.y, r.yy, -y3));
+    F2 s;
+    s.h = __fmul_rn(k.h, y3);
+    s.l = __fmaf_rn(k.h, y3, -s.h);
+    s.l = __fmaf_rn(k.l, y3, s.l);
+    s.l = __fmaf_rn(k.h, y3l, s.l);
+    s.l = __fmaf_rn(s.h, r.e * __fmaf_rn(1.875f, r.e, 1.5f), s.l);
+    return s;
+}
+
+// |a|^2 of a split vector
+__device__ __forceinline__ F2 f2_norm2(const F2 (&a)[3]) {
+    float p[3], q[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        p[c] = __fmul_rn(a[c].h, a[c].h);
+        q[c] = __fmaf_rn(a[c].h, a[c].h, -p[c]);
+        q[c] = __fmaf_rn(__fmaf_rn(2.0f, a[c].h, a[c].l), a[c].l, q[c]);
+    }
+    F2 r;
+    float e0, e1;
+    two_sum(p[0], p[1], r.h, e0);
+    two_sum(r.h, p[2], r.h, e1);
+    r.l = __fadd_rn(__fadd_rn(e0, e1), __fadd_rn(__fadd_rn(q[0], q[1]), q[2]));
+    return r;
 }
 
 // (a.x b.x + a.y b.y) + a.z b.z from split vectors.

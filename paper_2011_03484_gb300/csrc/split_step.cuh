@@ -26,18 +26,13 @@ struct SplitConsts {
     float rc2[kMaxPlanets];  // R_crit,j^2, rounded up by more than a float's error
 };
 
-__host__ __device__ inline F2 split_const(double x) {
-    const float h = (float)x;
-    return F2{h, (float)(x - (double)h)};
-}
-
 __host__ __device__ inline void split_planet(const ParticleConsts& pc, int j, SplitConsts& sc) {
-    sc.tg[j] = split_const(pc.tgm_full[j]);
+    sc.tg[j] = f2_const(pc.tgm_full[j]);
     sc.rc2[j] = (float)(pc.rc2[j] * (1.0 + 0x1p-20));
 }
 
 __host__ __device__ inline void split_step_consts(const ParticleConsts& pc, SplitConsts& sc) {
-    sc.dt = split_const(pc.dt);
+    sc.dt = f2_const(pc.dt);
     sc.mudt = pc.mu * pc.dt;
 }
 
@@ -187,35 +182,11 @@ constexpr float kSplitKick2 = 1.0f / 16384.0f;      // (2^-7)^2
 __device__ __forceinline__ bool kick_split(const F2 (&x)[3], const F2 (&P)[3], const F2& tg, float rc2, float lim2,
                                            F2 (&acc)[3]) {
     F2 d[3];
-    float p[3], q[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        float e;
-        two_sum(x[c].h, -P[c].h, d[c].h, e);
-        d[c].l = __fadd_rn(__fsub_rn(x[c].l, P[c].l), e);
-        p[c] = __fmul_rn(d[c].h, d[c].h);
-        q[c] = __fmaf_rn(d[c].h, d[c].h, -p[c]);
-        q[c] = __fmaf_rn(__fmaf_rn(2.0f, d[c].h, d[c].l), d[c].l, q[c]);
-    }
-    float D, e0, e1;
-    two_sum(p[0], p[1], D, e0);
-    two_sum(D, p[2], D, e1);
-    const float E = __fadd_rn(__fadd_rn(e0, e1), __fadd_rn(__fadd_rn(q[0], q[1]), q[2]));
-    // |d|^-3 = y^3 (1 - e)^(-3/2), e = 1 - |d|^2 y^2
-    const float y = rsqrt_f32(D);
-    const float yy = __fmul_rn(y, y), yl = __fmaf_rn(y, y, -yy);
-    float e = __fmaf_rn(-D, yy, 1.0f);
-    e = __fmaf_rn(-D, yl, e);
-    e = __fmaf_rn(-E, yy, e);
-    const float y3 = __fmul_rn(y, yy);
-    const float y3l = __fmaf_rn(y, yl, __fmaf_rn(y, yy, -y3));
-    F2 s;
-    s.h = __fmul_rn(tg.h, y3);
-    s.l = __fmaf_rn(tg.h, y3, -s.h);
-    s.l = __fmaf_rn(tg.l, y3, s.l);
-    s.l = __fmaf_rn(tg.h, y3l, s.l);
-    s.l = __fmaf_rn(s.h, e * __fmaf_rn(1.875f, e, 1.5f), s.l);
-    const bool far = (s.h * s.h <= lim2) && (D >= rc2);
+    for (int c = 0; c < 3; ++c) d[c] = f2_sub(x[c], P[c]);
+    const F2 D = f2_norm2(d);
+    F2 s = f2_k_rcube(f2_rsqrt(D), tg);
+    const bool far = (s.h * s.h <= lim2) && (D.h >= rc2);
     s.h = far ? s.h : 0.0f;
     s.l = far ? s.l : 0.0f;
 #pragma unroll
