@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(32) eph_setup_kernel(const double* __restrict_
 //   * warp 0 holds planet i in the four lanes 4i .. 4i + 3.  The drift's FP64
 //     arithmetic is the fast path of kepler.cuh with each instruction doing
 //     different things in a row's lanes (u and v^2; c2 and c3; F and r; the three
-//     components of x and v; ...): 33 FP64 instructions instead of ~66;
+//     components of x and v; ...): 31 FP64 instructions instead of ~66;
 //   * the kick is ~1e-3 of the velocity and is formed in float pairs
 //     (split_math.cuh) with lane 4i + c taking the interaction with planet j = c
 //     (and c + 4 for 5 to 8 planets); the star's part, which nearly cancels between
@@ -254,7 +254,7 @@ struct EphLane {
 
 // Limits of the pairs' kick: s = dt G m_j / |d|^3 against the orbit's rate (as in kick_split),
 // and |r|^2 / |q|^2 - 1 of the heliocentric and Jacobi positions.
-constexpr float kEphNear2 = 4.0e-6f;  // (0.002)^2
+constexpr float kEphNear2 = 1.6e-5f;  // (0.004)^2
 constexpr float kEphEps = 0.015625f;
 
 // The kick of a full step, dt dv/dt, for component min(col, 2) of the row's planet, at Jacobi
@@ -463,19 +463,21 @@ __device__ __forceinline__ void eph_dynamics(const PlanetConsts& pc, double* jac
         const double dot = fma(col == 0 ? q[0] : w[0], w[0],
                                fma(col == 0 ? q[1] : w[1], w[1], (col == 0 ? q[2] : w[2]) * w[2]));
         const double u = row_bc(dot, 0), v2 = row_bc(dot, 1);
-        const double beta = fma(2.0, mur0, -v2);
-        const double qq = fma(-beta, r0, mu);  // mu - beta r0
+        // beta = 2 mu/r0 - v^2, qq = mu - beta r0 = v^2 r0 - mu
+        const double bq = fma(odd ? v2 : 2.0, odd ? r0 : mur0, odd ? -mu : -v2);
+        const double beta = row_bc(bq, 0), qq = row_bc(bq, 1);
         const float r0f = d2f_bits(r0), uf = d2f_bits(u), bf = d2f_bits(beta), qf = d2f_bits(qq);
         const int er = exp_bits(r0), ev = exp_bits(v2);
         bool ok = er > 1023 - 60 && er < 1023 + 60 && ev < 1023 + 120 && ev > 1023 - 200;
         float sf, dsf = 0.f;
         {
-            // start: the series of s in dt to the third order
+            // start: the series of s in dt to the third order; then Newton steps, two for nearly
+            // circular orbits, until every planet's is below 2^-20 (five at most)
             const float ir = rcp_f32(r0f), h = dtf * ir, a = uf * h * ir;
             sf = h * fmaf(-1.0f / 6.0f * qf * ir, h * h, fmaf(0.5f * a, a - 1.0f, 1.0f));
         }
-#pragma unroll
-        for (int it = 0; it < 3; ++it) {
+#pragma unroll 1
+        for (int it = 0; it < 5; ++it) {
             const float s2f = sf * sf, zf = bf * s2f;
             const float c2 =
                 fmaf(zf, fmaf(zf, fmaf(zf, -1.0f / 40320.0f, 1.0f / 720.0f), -1.0f / 24.0f), 0.5f);
@@ -486,6 +488,7 @@ __device__ __forceinline__ void eph_dynamics(const PlanetConsts& pc, double* jac
             const float Fp = fmaf(r0f, fmaf(-zf, c2, 1.0f), fmaf(uf, G1, muf * G2));
             dsf = -F * rcp_f32(Fp);
             sf += dsf;
+            if (it >= 1 && __all_sync(kFullMask, !on || fabsf(dsf) <= 9.5367431640625e-7f * fabsf(sf))) break;
         }
         const float zf = bf * sf * sf;
         ok = ok && fabsf(zf) <= kZ7 && fabsf(dsf) <= 9.5367431640625e-7f * fabsf(sf) && isfinite(sf);
@@ -507,11 +510,11 @@ __device__ __forceinline__ void eph_dynamics(const PlanetConsts& pc, double* jac
         }
         const double W = (odd ? s3 : s2) * p;
         const double G2 = row_bc(W, 0), G3 = row_bc(W, 1);
-        const double G1 = fma(-beta, G3, s0);
-        // F (even columns) and r = T'(s)
-        double Fr = fma(odd ? 0.0 : mu, G3, odd ? r0 : -dt);
-        Fr = fma(odd ? qq : u, G2, Fr);
-        Fr = fma(odd ? u : r0, G1, Fr);
+        // even columns F = r0 s + qq G3 + u G2 - dt; odd G1 = s - beta G3 and r = T'(s) = r0 + u G1 + qq G2
+        double Fr = fma(odd ? -beta : u, odd ? G3 : G2, odd ? s0 : -dt);
+        const double G1 = row_bc(Fr, 1);
+        Fr = fma(odd ? u : qq, odd ? Fr : G3, odd ? r0 : Fr);
+        Fr = fma(odd ? qq : r0, odd ? G2 : s0, Fr);
         const double r = row_bc(Fr, 1);
         const F2 Fp = f2_split(row_bc(Fr, 0)), rp = f2_split(r);
         // Halley step dH = dN (1 - dN T''/(2 T')), dN = -F / r (a pair: dN is below 2^-20 s)
@@ -519,14 +522,12 @@ __device__ __forceinline__ void eph_dynamics(const PlanetConsts& pc, double* jac
         const F2 dN = f2_div(F2{-Fp.h, -Fp.l}, rp, ri);
         const float G2f = d2f_bits(G2), G1f = d2f_bits(G1), G0f = fmaf(-bf, G2f, 1.0f);
         const float kf = 0.5f * dN.h * fmaf(uf, G0f, qf * G1f) * ri;
-        const double dH = f2_double(f2_norm(dN.h, fmaf(-dN.h, kf, dN.l)));
-        ok = ok && (__double2hiint(r) > 0) && (exp_bits(dH) + 14 <= exp_bits(s0) || dH == 0.0);
-        const float hf = 0.5f * dN.h;
-        // G2(s + d) = G2 + d (G1 + d/2 G0), G3 + d (G2 + d/2 G1); column 2: s + d
-        double tn = (odd ? G2 : G1) + f2d_bits(hf * (odd ? G1f : G0f));
-        tn = fma(dH, col == 2 ? 1.0 : tn, col == 2 ? s0 : (odd ? G3 : G2));
-        const double G2n = row_bc(tn, 0), G3n = row_bc(tn, 1);
-        const double G1n = fma(-beta, G3n, row_bc(tn, 2));
+        // G2(s + dH) = G2 + dH G1 (1 + dH G0 / (2 G1)), G3 + dH G2 (1 + dH G1 / (2 G2)); column 2: s + dH
+        const float hf = 0.5f * dN.h * (odd ? G1f * rcp_f32(G2f) : G0f * rcp_f32(G1f));
+        const double dl = f2_double(f2_norm(dN.h, fmaf(dN.h, (col == 2 ? 0.0f : hf) - kf, dN.l)));
+        const double Gn = fma(dl, col == 2 ? 1.0 : (odd ? G2 : G1), col == 2 ? s0 : (odd ? G3 : G2));
+        ok = ok && (__double2hiint(r) > 0) && fabsf(dN.h) <= 6.1035156e-5f * fabsf(sf);
+        const double G2n = row_bc(Gn, 0), G3n = row_bc(Gn, 1);
         const double fg = fma(odd ? -mu : -mur0, odd ? G3n : G2n, odd ? dt : 0.0);  // f - 1, g
         const double fm1 = row_bc(fg, 0), g = row_bc(fg, 1);
         const double qc = own(q);
@@ -548,6 +549,7 @@ __device__ __forceinline__ void eph_dynamics(const PlanetConsts& pc, double* jac
         // |x|, mu/|x| of the new position; fdot, gdot - 1
         const double x2 = fma(qnew[0], qnew[0], fma(qnew[1], qnew[1], qnew[2] * qnew[2]));
         const double rinv = rsqrt_full(x2);
+        const double G1n = fma(-beta, G3n, row_bc(Gn, 2));
         const double m1 = (col == 0 ? mur0 : (col == 1 ? mu : x2)) * rinv;
         const double m2 = -m1 * (col == 0 ? G1n : G2n);
         const double fd = row_bc(m2, 0), gdm1 = row_bc(m2, 1);

@@ -98,23 +98,26 @@ __device__ __forceinline__ int kick_near(unsigned near, double x, double y, doub
 
 // The kick of a full step, K = dt a(r) at log step L (a half kick is exactly half
 // of it), and the encounter test: h0 and the planets in pairs (kick_split), in
-// FP64 the planets a lane is near to, and the whole sum where it exceeds 2^-7 |v|
+// FP64 (N) the planets a lane is near to, and the whole sum where it exceeds 2^-7 |v|
 // (far out, where h0 outweighs the star: a pair's 46 bits of K would show in v).
+// base: the part of the drift's velocity still in pairs; on return C = base + K - N.
 // X: the position split; sp.v2 is negative where the position is out of the
 // floats' range (then all is FP64).  Returns the lowest 1-based planet index whose
-// test fires, or 0.  All lanes of a warp call it together.
+// test fires, or 0; *exact: some lane's N is not zero.  All lanes of a warp call it
+// together.
 // TPP = 2: a lane pair (both lanes holding the same particle) splits the planets:
 // lane parity p takes planets p, p + 2, ..., the partial sums are added (the
 // same bits on both lanes: two_sum and addition commute) and the lower index wins.
 template <int NP, int TPP>
-__device__ __forceinline__ int kick_sum(double x, double y, double z, const F2 (&X)[3], const Speed& sp, bool act,
-                                        const double* __restrict__ L, const ParticleConsts& pc, const SplitConsts& sc,
-                                        double (&K)[3]) {
+__device__ __forceinline__ int kick_sum(double x, double y, double z, const F2 (&X)[3], const F2 (&base)[3],
+                                        const Speed& sp, bool act, const double* __restrict__ L,
+                                        const ParticleConsts& pc, const SplitConsts& sc, F2 (&C)[3], double (&N)[3],
+                                        bool& exact) {
     const int parity = TPP == 2 ? (int)(threadIdx.x & 1) : 0;
     const float lim2 = kSplitNear2 * sp.rate2;
-    F2 acc[3];
-    load_rec_split(L + kRec * NP, acc);
-    if (TPP == 2 && parity == 1) acc[0] = acc[1] = acc[2] = F2{0.0f, 0.0f};
+    load_rec_split(L + kRec * NP, C);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) C[c] = TPP == 2 && parity == 1 ? F2{0.0f, 0.0f} : f2_add(base[c], C[c]);
     unsigned near = 0, mine = parity == 0 ? 1u << NP : 0u;
 #pragma unroll
     for (int jj = (NP + TPP - 1) / TPP - 1; jj >= 0; --jj) {
@@ -122,45 +125,48 @@ __device__ __forceinline__ int kick_sum(double x, double y, double z, const F2 (
         if (j < NP) {
             F2 P[3];
             load_rec_split(L + kRec * j, P);
-            if (!kick_split(X, P, sc.tg[j], sc.rc2[j], lim2, acc)) near |= 1u << j;
+            if (!kick_split(X, P, sc.tg[j], sc.rc2[j], lim2, C)) near |= 1u << j;
             mine |= 1u << j;
         }
     }
     if constexpr (TPP == 2) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float oh = __shfl_xor_sync(kFullMask, acc[c].h, 1), ol = __shfl_xor_sync(kFullMask, acc[c].l, 1);
-            float e;
-            two_sum(acc[c].h, oh, acc[c].h, e);
-            acc[c].l = __fadd_rn(e, __fadd_rn(acc[c].l, ol));
-        }
+        for (int c = 0; c < 3; ++c)
+            C[c] = f2_add(C[c], F2{__shfl_xor_sync(kFullMask, C[c].h, 1), __shfl_xor_sync(kFullMask, C[c].l, 1)});
     }
-    const float k2 = fmaf(acc[0].h, acc[0].h, fmaf(acc[1].h, acc[1].h, acc[2].h * acc[2].h));
+    const float k2 = fmaf(C[0].h, C[0].h, fmaf(C[1].h, C[1].h, C[2].h * C[2].h));
     const bool small = k2 <= kSplitKick2 * sp.v2;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) K[c] = f2_double(f2_norm(acc[c].h, acc[c].l));
     int hit = 0;
-    if (__any_sync(kFullMask, act && (near != 0u || !small))) {
+    exact = __any_sync(kFullMask, act && (near != 0u || !small));
+    if (exact) {
+        N[0] = N[1] = N[2] = 0.0;
         if (!small) {
             near = mine;
-            K[0] = K[1] = K[2] = 0.0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) C[c] = base[c];
         }
         if (!act) near = 0;
+        if (TPP == 2 || near) hit = kick_near<NP>(near, x, y, z, L, pc, N);
         if constexpr (TPP == 2) {
-            double N[3] = {0.0, 0.0, 0.0};
-            hit = kick_near<NP>(near, x, y, z, L, pc, N);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) K[c] += N[c] + __shfl_xor_sync(kFullMask, N[c], 1);
+            for (int c = 0; c < 3; ++c) N[c] += __shfl_xor_sync(kFullMask, N[c], 1);
             const int other = __shfl_xor_sync(kFullMask, hit, 1);
             hit = (hit != 0 && other != 0) ? min(hit, other) : (hit | other);
-        } else if (near) {
-            hit = kick_near<NP>(near, x, y, z, L, pc, K);
         }
     }
     return hit;
 }
 
-// The FP64 drift (kepler.cuh) of the lanes that drift_split leaves (part): the fast
+__device__ __forceinline__ double f2_sum(const F2& v) { return f2_double(f2_norm(v.h, v.l)); }
+
+// drift_wide out of line (few warps need it: its registers and code stay off the usual path).
+static __device__ __noinline__ bool drift_wide_call(double r2, double mudt, double dt, F2 dt2, double x, double y,
+                                                    double z, double vx, double vy, double vz, DriftFactors& f) {
+    const double s[6] = {x, y, z, vx, vy, vz};
+    return drift_wide(r2, mudt, dt, dt2, s, f);
+}
+
+// The FP64 drift (kepler.cuh) of the lanes that the pairs leave (part): the fast
 // path, then the general solver for lanes outside its domain.  Returns false for a
 // lane whose solve failed.  All lanes of a warp call it together.
 static __device__ __noinline__ bool drift_fp64(const ParticleConsts& pc, bool part, double (&s)[6]) {
@@ -229,33 +235,58 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
     }
     F2 X[3] = {f2_split(x), f2_split(y), f2_split(z)};
     double r2 = fma(x, x, fma(y, y, z * z));
+    constexpr F2 kZero = {0.0f, 0.0f};
     if (!open_in) {
-        double K[3];
-        kick_sum<NP, TPP>(x, y, z, X, float_speed(r2, vx, vy, vz), act, L, pc, sc, K);
+        const F2 base[3] = {kZero, kZero, kZero};
+        F2 C[3];
+        double N[3];
+        bool exact;
+        kick_sum<NP, TPP>(x, y, z, X, base, float_speed(r2, vx, vy, vz), act, L, pc, sc, C, N, exact);
         if (act) {
-            vx = fma(0.5, K[0], vx);
-            vy = fma(0.5, K[1], vy);
-            vz = fma(0.5, K[2], vz);
+            vx = fma(0.5, f2_sum(C[0]), vx);
+            vy = fma(0.5, f2_sum(C[1]), vy);
+            vz = fma(0.5, f2_sum(C[2]), vz);
+            if (exact) {
+                vx = fma(0.5, N[0], vx);
+                vy = fma(0.5, N[1], vy);
+                vz = fma(0.5, N[2], vz);
+            }
         }
     }
 
     for (int k = 0; k < nsteps; ++k) {
         if (!__any_sync(kFullMask, act)) break;
         const double* __restrict__ Ln = L + (size_t)(k + 1) * S;
+        // the drifted position n[0..2] and velocity n[3..5] + base: (gdot - 1) v stays in pairs,
+        // to enter the velocity in one sum with the kick
         double n[6];
+        F2 base[3] = {kZero, kZero, kZero};
         bool failed = false;
         Speed sp;
         if constexpr (MODE == kDriftConverge) {
             const F2 V[3] = {f2_split(vx), f2_split(vy), f2_split(vz)};
             DriftFactors f;
-            const bool fast = drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp) && act;
+            bool slow = !drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp) && act;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) base[c] = f2_mul(f.gdm1, V[c]);
+            if (__any_sync(kFullMask, slow)) {
+                DriftFactors w;
+                const bool done = drift_wide_call(r2, sc.mudt, pc.dt, sc.dt, x, y, z, vx, vy, vz, w);
+                if (slow && done) {
+                    slow = false;
+                    f.fm1 = w.fm1;
+                    f.g = w.g;
+                    f.fd = w.fd;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) base[c] = f2_muln(w.gdm1, f2_normp(V[c]));
+                }
+            }
             n[0] = fma(f.fm1, x, fma(f.g, vx, x));
             n[1] = fma(f.fm1, y, fma(f.g, vy, y));
             n[2] = fma(f.fm1, z, fma(f.g, vz, z));
-            n[3] = fma(f.fd, x, fma(f.gdm1, vx, vx));
-            n[4] = fma(f.fd, y, fma(f.gdm1, vy, vy));
-            n[5] = fma(f.fd, z, fma(f.gdm1, vz, vz));
-            const bool slow = act && !fast;
+            n[3] = fma(f.fd, x, vx);
+            n[4] = fma(f.fd, y, vy);
+            n[5] = fma(f.fd, z, vz);
             if (__any_sync(kFullMask, slow)) {
                 double s[6] = {x, y, z, vx, vy, vz};
                 const bool done = drift_fp64(pc, slow, s);
@@ -263,6 +294,7 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
                     failed = !done;
 #pragma unroll
                     for (int c = 0; c < 6; ++c) n[c] = s[c];
+                    base[0] = base[1] = base[2] = kZero;
                 }
             }
         } else {
@@ -300,34 +332,54 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
         // escape: |r|^2 > r_max^2 (integer compare of non-negative doubles)
         int hit = (__double_as_longlong(pc.rmax2) != 0 && lt_nonneg(pc.rmax2, r2)) ? GLISSE_REMOVED_ESCAPE : 0;
         if (!in_float_range(r2)) sp.v2 = -1.0f;
-        double K[3];
-        const int enc = kick_sum<NP, TPP>(x, y, z, X, sp, act, Ln, pc, sc, K);
+        F2 C[3];
+        double N[3];
+        bool exact;
+        const int enc = kick_sum<NP, TPP>(x, y, z, X, base, sp, act, Ln, pc, sc, C, N, exact);
         hit = enc ? enc : hit;
         const bool last = k + 1 == nsteps;
-        if constexpr (PUBLISH) {
-            if (pub.out && !close_out && last && act && hit == 0) {
-                double* o = pub.out + 6 * (int64_t)pub.id[pub.slot];
-                o[0] = x;
-                o[1] = y;
-                o[2] = z;
-                o[3] = fma(0.5, K[0], vx);
-                o[4] = fma(0.5, K[1], vy);
-                o[5] = fma(0.5, K[2], vz);
+        if (last) {
+            // the synchronised state: drift and half of the kick, base + K/2 = (base + C) / 2
+            if (act && hit == 0 && (close_out || (PUBLISH && pub.out))) {
+                double h[3] = {vx, vy, vz};
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    h[c] = fma(0.5, f2_sum(f2_add(base[c], C[c])), h[c]);
+                    if (exact) h[c] = fma(0.5, N[c], h[c]);
+                }
+                if (close_out) {
+                    vx = h[0];
+                    vy = h[1];
+                    vz = h[2];
+                    break;
+                }
+                if constexpr (PUBLISH) {
+                    double* o = pub.out + 6 * (int64_t)pub.id[pub.slot];
+                    o[0] = x;
+                    o[1] = y;
+                    o[2] = z;
+                    o[3] = h[0];
+                    o[4] = h[1];
+                    o[5] = h[2];
+                }
             }
         }
         if (act) {
+            // a removed particle keeps the drifted velocity
             if (hit != 0) {
                 act = false;
                 reason = hit;
                 rstep = step0 + k + 1;
-            } else if (close_out && last) {
-                vx = fma(0.5, K[0], vx);
-                vy = fma(0.5, K[1], vy);
-                vz = fma(0.5, K[2], vz);
-            } else {
-                vx += K[0];
-                vy += K[1];
-                vz += K[2];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) C[c] = base[c];
+            }
+            vx += f2_sum(C[0]);
+            vy += f2_sum(C[1]);
+            vz += f2_sum(C[2]);
+            if (exact && act) {
+                vx += N[0];
+                vy += N[1];
+                vz += N[2];
             }
         }
     }
@@ -350,7 +402,8 @@ __device__ __forceinline__ void store_removed(int64_t pid, double x, double y, d
 
 template <int NP, int MODE>
 __global__ void __launch_bounds__(kParticleBlock, GLISSE_PARTICLE_MIN_BLOCKS)
-    particle_chunk_kernel(const ChunkArgs a, const ParticleConsts pc, const SplitConsts sc) {
+    particle_chunk_kernel(const ChunkArgs a, const __grid_constant__ ParticleConsts pc,
+                          const __grid_constant__ SplitConsts sc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool in = i < a.n;
     const int64_t ld = a.ld;
@@ -440,7 +493,8 @@ constexpr int kTaskMaxBlocks = 4;
 
 template <int NP>
 __global__ void __launch_bounds__(kParticleBlock, kTaskMaxBlocks)
-    particle_tasks_kernel(const ChunkArgs a, const ParticleConsts pc, const SplitConsts sc, const TaskArgs ta) {
+    particle_tasks_kernel(const ChunkArgs a, const __grid_constant__ ParticleConsts pc,
+                          const __grid_constant__ SplitConsts sc, const TaskArgs ta) {
     const int lane = threadIdx.x & 31;
     const int64_t ld = a.ld;
     const int S = log_stride(NP);

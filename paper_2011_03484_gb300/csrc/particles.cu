@@ -60,7 +60,7 @@ __device__ __forceinline__ void batch_task(const BatchArgs& a, const ParticleCon
 constexpr int kBatchMaxWarps = 8;  // largest block of the batched kernel: 256 threads
 
 template <int TPP>
-__global__ void __launch_bounds__(32 * kBatchMaxWarps) batch_particle_kernel(const BatchArgs a) {
+__global__ void __launch_bounds__(32 * kBatchMaxWarps, 2) batch_particle_kernel(const BatchArgs a) {
     __shared__ ParticleConsts s_pc[kBatchMaxWarps];
     __shared__ SplitConsts s_sc[kBatchMaxWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -66,6 +66,15 @@ __device__ __forceinline__ F2 f2_mul(const F2& a, const F2& b) {
     return r;
 }
 
+// Product, normalised, of normalised pairs: to 2^-48.
+__device__ __forceinline__ F2 f2_muln(const F2& a, const F2& b) {
+    const float h = __fmul_rn(a.h, b.h);
+    const float t = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmul_rn(a.l, b.l)));
+    return f2_norm(h, __fadd_rn(__fmaf_rn(a.h, b.h, -h), t));
+}
+
+__device__ __forceinline__ F2 f2_normp(const F2& a) { return f2_norm(a.h, a.l); }
+
 __device__ __forceinline__ F2 f2_add(const F2& a, const F2& b) {
     F2 r;
     float e;
@@ -90,6 +99,16 @@ __device__ __forceinline__ F2 f2_div(const F2& a, const F2& b, float rb) {
     e = __fadd_rn(__fmaf_rn(-q.h, b.l, e), a.l);
     q.l = __fmul_rn(e, rb);
     return q;
+}
+
+// The same, normalised, to 2^-48.
+__device__ __forceinline__ F2 f2_divn(const F2& a, const F2& b, float rb) {
+    const float q = __fmul_rn(a.h, rb);
+    const float e = __fadd_rn(__fmaf_rn(-q, b.l, __fmaf_rn(-q, b.h, a.h)), a.l);
+    const float l = __fmul_rn(e, rb);
+    F2 r = f2_norm(q, l);
+    r.l = __fmaf_rn(__fmaf_rn(-l, b.h, e), rb, r.l);
+    return r;
 }
 
 // a - b c
@@ -151,6 +170,16 @@ __device__ __forceinline__ F2 f2_dot(const F2 (&a)[3], const F2 (&b)[3]) {
     return s;
 }
 
+// f2_dot with normalised products.
+__device__ __forceinline__ F2 f2_dotn(const F2 (&a)[3], const F2 (&b)[3]) {
+    const F2 p = f2_muln(a[0], b[0]), q = f2_muln(a[1], b[1]), r = f2_muln(a[2], b[2]);
+    F2 s;
+    float e, f;
+    two_sum(p.h, q.h, s.h, e);
+    two_sum(s.h, r.h, s.h, f);
+    return f2_norm(s.h, __fadd_rn(__fadd_rn(e, f), __fadd_rn(__fadd_rn(p.l, q.l), r.l)));
+}
+
 // A double as a pair, by integer operations and one int-to-float conversion
 // (an F2F conversion occupies the FP64 pipe): the leading 24 bits, and the other
 // 29 rounded to 24.  |x| below 2^-74 is read as 2^-74 (1 + ...): far below
@@ -163,6 +192,54 @@ __device__ __forceinline__ F2 f2_split(double x) {
     r.h = __uint_as_float(b);
     r.l = __fmul_rn((float)(int)(lo & 0x1FFFFFFFu), __uint_as_float((b & 0xFF800000u) - (52u << 23)));
     return r;
+}
+
+// A positive double's leading 24 bits (truncated) as a float; x in the float's normal range.
+__device__ __forceinline__ float f32_trunc(double x) {
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)__double2hiint(x), 3) + 0x40000000u);
+}
+
+// y^2 exactly for a float y of at most 21 significant bits (in [2^-60, 2^60]).
+__device__ __forceinline__ double f21_square(float y) {
+    const unsigned b = __float_as_uint(y);
+    const unsigned m = ((b & 0x7FFFFFu) | 0x800000u) >> 3;       // y = m 2^(ey - 147)
+    const unsigned long long m2 = (unsigned long long)m * m;     // [2^40, 2^42)
+    const int a = (int)(m2 >> 41);
+    return __longlong_as_double(((long long)(2 * (int)(b >> 23) + 768 + a) << 52) + (long long)(m2 << (12 - a)));
+}
+
+// f2_split with the leading part rounded to nearest: the rest, and its rounding error,
+// are half as large (four instructions more).
+__device__ __forceinline__ F2 f2_split_near(double x) {
+    const unsigned lo = (unsigned)__double2loint(x), hi = (unsigned)__double2hiint(x);
+    const unsigned long long a =
+        ((unsigned long long)max(hi & 0x7FFFFFFFu, (unsigned)(1023 - 74) << 20) << 32) | lo;
+    const unsigned long long r = a + 0x10000000ull;
+    const unsigned sign = hi & 0x80000000u;
+    F2 v;
+    v.h = __uint_as_float((__funnelshift_l((unsigned)r, (unsigned)(r >> 32), 3) + 0x40000000u) | sign);
+    // the 29 low bits as a signed number, in units of 2^-55 of x's binade
+    const unsigned sc = ((((unsigned)(a >> 32) << 3) & 0xFF800000u) + 0x40000000u - (55u << 23)) | sign;
+    v.l = __fmul_rn((float)(int)(lo << 3), __uint_as_float(sc));
+    return v;
+}
+
+// k y^3 correctly rounded (ties away from zero) for a float y > 0 of at most 21 significant
+// bits, by integer arithmetic as in seed_square_kcube; its range check is the caller's
+// (y in [2^-60, 2^60], k normal).
+__device__ __forceinline__ double f21_kcube(float y, double k) {
+    const unsigned b = __float_as_uint(y);
+    const int ey = (int)(b >> 23);                              // y = m 2^(ey - 147)
+    const unsigned m = ((b & 0x7FFFFFu) | 0x800000u) >> 3;     // [2^20, 2^21)
+    const unsigned long long m3 = (unsigned long long)m * m * m;  // [2^60, 2^63)
+    const long long kb = __double_as_longlong(k);
+    const int ek = (int)((kb >> 52) & 0x7FF);
+    const unsigned long long km = ((unsigned long long)kb & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const unsigned long long p = __umul64hi(km << 11, m3 << 1);
+    const int sh = 11 - __clzll(p);
+    const unsigned long long q = ((p >> (sh - 1)) + 1) >> 1;
+    const int be = sh + ek + 3 * (ey + 896) - 3077;
+    return __longlong_as_double((((long long)(be - 1) << 52) + (long long)q) | (kb & (long long)(1ull << 63)));
 }
 
 // A normalised pair (|l| <= ulp(h)) as a double: h's bits moved to a double,
