@@ -84,12 +84,12 @@ extern "C" {
 /* launch shape of the particle map (results are bit-identical in every shape).
  * PLAIN: one thread per particle slot, one launch per segment.  TASKS: a
  * persistent grid of a few warps per SM partition that take (32-slot group,
- * 32-step sub-chunk) tasks in order from a device counter, so every partition
- * keeps the same number of busy warps to the end of the segment; a task waits
- * (bounded: GLISSE_E_TIMEOUT after seconds) for its group's previous
- * sub-chunk.  AUTO picks TASKS when the live groups outnumber the resident
- * warps (two to four per partition) by half again, PLAIN otherwise.  The
- * fixed-iteration Kepler mode always uses PLAIN. */
+ * 32-step sub-chunk) tasks by tickets from a device counter, first every group's first
+ * sub-chunk and then whichever group is ready, so every partition
+ * keeps the same number of busy warps to the end of the segment; a warp without a
+ * ready task waits (bounded: GLISSE_E_TIMEOUT after seconds).  AUTO picks TASKS when
+ * the live groups outnumber the resident warps (two to five per partition) by a
+ * quarter, PLAIN otherwise.  The fixed-iteration Kepler mode always uses PLAIN. */
 #define GLISSE_LAUNCH_AUTO 0
 #define GLISSE_LAUNCH_PLAIN 1
 #define GLISSE_LAUNCH_TASKS 2

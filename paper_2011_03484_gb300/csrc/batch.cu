@@ -5,8 +5,9 @@
 // decreasing planet count (the costliest tasks are handed out first, which
 // keeps the persistent kernel's tail short).  One chunk is:
 //   1. eph_batch_kernel      planet chunk of every system (block = system)
-//   2. batch_particle_kernel persistent; warps take 32-particle tasks, one lane
-//                            (or, chosen by the autotuner, a lane pair) per particle
+//   2. batch_particle_kernel persistent; warps take tasks of 32 particles over a
+//                            sub-chunk of steps, one lane (or, chosen by the
+//                            autotuner, a lane pair) per particle
 //   3. stable partition      count / scan / scatter, sizes read on the device
 //   4. flags + task rebuild  per-system live counts -> offsets -> task table,
 //                            clock advanced
@@ -256,6 +257,7 @@ struct glisse_batch {
     int64_t max_tasks = 0;
     int64_t* d_n_tasks = nullptr;
     int* d_counter = nullptr;
+    uint32_t* d_queue = nullptr;  // groups ready for their next sub-chunk (particle kernel)
     BatchClock* d_clock = nullptr;
     int64_t* d_nlive = nullptr;
     int64_t* d_nkept = nullptr;
@@ -303,7 +305,7 @@ static void batch_free(glisse_batch* b) {
     void* ptrs[] = {b->d_pcs, b->d_ppcs, b->d_np, b->d_jac, b->d_dt, b->d_log, b->d_log_off, b->d_status,
                     b->d_st[0], b->d_st[1], b->d_id[0], b->d_id[1], b->d_alive, b->d_out_state, b->d_out_step,
                     b->d_out_reason, b->d_cnt, b->d_task_sys, b->d_task_start, b->d_task_count, b->d_n_tasks,
-                    b->d_counter, b->d_clock, b->d_nlive, b->d_nkept, b->d_counts, b->d_steps};
+                    b->d_counter, b->d_queue, b->d_clock, b->d_nlive, b->d_nkept, b->d_counts, b->d_steps};
     for (void* p : ptrs) cudaFree(p);
     for (cudaEvent_t e : b->ev)
         if (e) cudaEventDestroy(e);
@@ -349,6 +351,8 @@ static int enqueue_chunk(glisse_batch* b, int m) {
     a.task_count = b->d_task_count;
     a.n_tasks = b->d_n_tasks;
     a.counter = b->d_counter;
+    a.queue = b->d_queue;
+    a.status = b->d_status;
     a.clock = b->d_clock;
     a.ld = b->cap;
     a.st = b->d_st[b->cur];
@@ -360,6 +364,7 @@ static int enqueue_chunk(glisse_batch* b, int m) {
     a.out_step = b->d_out_step;
     a.out_reason = b->d_out_reason;
     a.steps_done = b->d_steps;
+    GB_CUDA(cudaMemsetAsync(b->d_queue, 0, sizeof(uint32_t) * task_queue_words(32 * b->max_tasks), s));
     GB_CUDA(launch_batch_particles(a, b->blocks, b->threads, b->tpp, s));
     if (b->timing) GB_CUDA(cudaEventRecord(b->ev[2], s));
     const unsigned tiles = (unsigned)((b->cap + kBTile - 1) / kBTile);
@@ -480,6 +485,7 @@ static int batch_alloc(glisse_batch* b, std::vector<int64_t>& log_off) {
     GB_ALLOC(b->d_task_count, sizeof(int32_t) * b->max_tasks);
     GB_ALLOC(b->d_n_tasks, sizeof(int64_t));
     GB_ALLOC(b->d_counter, sizeof(int));
+    GB_ALLOC(b->d_queue, sizeof(uint32_t) * task_queue_words(32 * b->max_tasks));
     GB_ALLOC(b->d_clock, sizeof(BatchClock));
     GB_ALLOC(b->d_nlive, sizeof(int64_t));
     GB_ALLOC(b->d_nkept, sizeof(int64_t));

@@ -149,7 +149,7 @@ struct glisse_ctx {
     unsigned long long* d_steps = nullptr;   // exact particle-step counter (timing mode)
     unsigned long long* h_steps = nullptr;
     unsigned long long* d_task = nullptr;    // task counter of the particle kernel's task mode
-    int32_t* d_group_done = nullptr;         // [ceil(cap / 32)] sub-chunks finished per 32-slot group
+    uint32_t* d_queue = nullptr;             // and its queue of groups ready for their next sub-chunk
     unsigned long long* d_live = nullptr;    // particles live at the end of the last segment
     unsigned long long* h_live = nullptr;
     int64_t n_alive = 0;                     // live particles (n_live counts slots, dead ones included
@@ -471,7 +471,7 @@ static int setup(glisse_ctx* c, const double* planets, const double* particles, 
                      o_counts = take(sizeof(int64_t) * (size_t)compact_scratch_entries(cap)),
                      o_nlive = take(sizeof(int64_t)), o_steps = take(sizeof(unsigned long long)),
                      o_live = take(sizeof(unsigned long long)), o_task = take(sizeof(unsigned long long)),
-                     o_groups = take(sizeof(int32_t) * (size_t)((cap + 31) / 32));
+                     o_queue = take(sizeof(uint32_t) * task_queue_words(cap));
         GL_ALLOC(c->d_arena, off);
         char* base = static_cast<char*>(c->d_arena);
         c->d_pc = reinterpret_cast<PlanetConsts*>(base + o_pc);
@@ -499,7 +499,7 @@ static int setup(glisse_ctx* c, const double* planets, const double* particles, 
         c->d_steps = c->timing ? reinterpret_cast<unsigned long long*>(base + o_steps) : nullptr;
         c->d_live = reinterpret_cast<unsigned long long*>(base + o_live);
         c->d_task = reinterpret_cast<unsigned long long*>(base + o_task);
-        c->d_group_done = reinterpret_cast<int32_t*>(base + o_groups);
+        c->d_queue = reinterpret_cast<uint32_t*>(base + o_queue);
     }
     for (Slot& sl : c->ring)
         if (!alloc_slot(c, sl)) return GLISSE_E_NOMEM;
@@ -882,7 +882,7 @@ extern "C" int glisse_advance(glisse_ctx* c, int64_t n_steps) {
             a.live_out = c->d_live;
             TaskArgs tasks{};
             tasks.task_counter = c->d_task;
-            tasks.group_done = c->d_group_done;
+            tasks.queue = c->d_queue;
             tasks.status = c->d_status;
 
             GL_CUDA(cudaMemsetAsync(c->d_live, 0, sizeof(unsigned long long), c->s));

@@ -99,17 +99,18 @@ struct ChunkArgs {
 };
 
 // Task mode of the particle kernel (particle_tasks_kernel): the segment is cut into
-// sub-chunks of sub_steps steps; task t = (group t mod n_groups, sub-chunk t / n_groups),
-// where a group is the 32 slots one warp holds, is taken in order from task_counter by
-// persistent warps.  (A separate argument: the plain kernel's registers are tight.)
+// sub-chunks of sub_steps steps; a task is a group (the 32 slots one warp holds) over
+// one sub-chunk.  (A separate argument: the plain kernel's registers are tight.)
 struct TaskArgs {
     int32_t sub_steps;                 // steps per sub-chunk
     int32_t n_groups;                  // ceil(n / 32)
-    unsigned long long* task_counter;  // zero before the launch
-    int32_t* group_done;               // [n_groups] sub-chunks of each group finished; zero before the launch
-    int* status;                       // set to GLISSE_E_TIMEOUT if a wait for a group gives up
+    unsigned long long* task_counter;  // tickets taken; zero before the launch
+    uint32_t* queue;                   // [2 + n_groups (n_sub - 1)] counts and entries; zero before the launch
+    int* status;                       // set to GLISSE_E_TIMEOUT if a wait for the queue gives up
     int32_t wait_polls;                // polls before a wait gives up; 0: the default (seconds)
 };
+// entries that holds for any segment of n slots (at most 31 sub-chunks after a group's first)
+inline size_t task_queue_words(int64_t n) { return 2 + 31 * (size_t)((n + 31) / 32); }
 
 // Device-resident clock of a batch (so a captured chunk graph can be replayed).
 struct BatchClock {
@@ -118,7 +119,7 @@ struct BatchClock {
     int32_t pad;
 };
 
-// Arguments of the persistent batched particle kernel.  Task t covers
+// Arguments of the persistent batched particle kernel.  Group t covers
 // particles [task_start[t], task_start[t] + task_count[t]) of system task_sys[t]
 // (task_count <= 32: one warp).
 struct BatchArgs {
@@ -130,7 +131,9 @@ struct BatchArgs {
     const int64_t* task_start;
     const int32_t* task_count;
     const int64_t* n_tasks;     // device scalar
-    int* counter;               // work counter, zero before the launch
+    int* counter;               // tickets taken, zero before the launch
+    uint32_t* queue;            // [2 + 31 max tasks] as TaskArgs::queue, zero before the launch
+    int* status;                // set to GLISSE_E_TIMEOUT if a wait for the queue gives up
     const BatchClock* clock;
     int64_t ld;
     double* st;                 // [6][ld]

@@ -49,6 +49,7 @@ constexpr int kParticleBlock = 128;
 // paper's fixed-iteration solve (GLISSE_KEPLER_PAPER_FIXED)
 constexpr int kDriftConverge = 0;
 constexpr int kDriftPaper = 1;
+constexpr int kAnyNp = -1;  // planet count at run time
 
 // Read-only broadcast loads of one log record: its doubles, and its pairs.
 __device__ __forceinline__ void load_rec(const double* __restrict__ p, double& x, double& y, double& z) {
@@ -66,22 +67,21 @@ __device__ __forceinline__ void load_rec_split(const double* __restrict__ p, F2 
     v[2] = F2{a.z, b.y};
 }
 
-// The terms that kick_sum leaves to FP64 (bit j of `near`: planet j, bit NP: h0), for
+// The terms that kick_sum leaves to FP64 (bit j of `near`: planet j, bit np: h0), for
 // one lane: added to K, with the encounter test.  Returns the lowest 1-based
 // planet index whose test fires, or 0.
-template <int NP>
-__device__ __forceinline__ int kick_near(unsigned near, double x, double y, double z, const double* __restrict__ L,
-                                      const ParticleConsts& pc, double (&K)[3]) {
+__device__ __forceinline__ int kick_near(unsigned near, int np, double x, double y, double z,
+                                         const double* __restrict__ L, const ParticleConsts& pc, double (&K)[3]) {
     int hit = 0;
-    if ((near >> NP) & 1u) {
+    if ((near >> np) & 1u) {
         double hx, hy, hz;
-        load_rec(L + kRec * NP, hx, hy, hz);
+        load_rec(L + kRec * np, hx, hy, hz);
         K[0] = fma(pc.dt, hx, K[0]);
         K[1] = fma(pc.dt, hy, K[1]);
         K[2] = fma(pc.dt, hz, K[2]);
     }
 #pragma unroll 1
-    for (int j = NP - 1; j >= 0; --j) {
+    for (int j = np - 1; j >= 0; --j) {
         if (!((near >> j) & 1u)) continue;
         double px, py, pz;
         load_rec(L + kRec * j, px, py, pz);
@@ -108,21 +108,24 @@ __device__ __forceinline__ int kick_near(unsigned near, double x, double y, doub
 // TPP = 2: a lane pair (both lanes holding the same particle) splits the planets:
 // lane parity p takes planets p, p + 2, ..., the partial sums are added (the
 // same bits on both lanes: two_sum and addition commute) and the lower index wins.
+// NP: the planet count, or kAnyNp to take it from np_any (one code for all counts).
 template <int NP, int TPP>
-__device__ __forceinline__ int kick_sum(double x, double y, double z, const F2 (&X)[3], const F2 (&base)[3],
-                                        const Speed& sp, bool act, const double* __restrict__ L,
+__device__ __forceinline__ int kick_sum(int np_any, double x, double y, double z, const F2 (&X)[3],
+                                        const F2 (&base)[3], const Speed& sp, bool act, const double* __restrict__ L,
                                         const ParticleConsts& pc, const SplitConsts& sc, F2 (&C)[3], double (&N)[3],
                                         bool& exact) {
+    const int np = NP >= 0 ? NP : np_any;
+    constexpr int kUnroll = NP >= 0 ? kMaxPlanets : 2;
     const int parity = TPP == 2 ? (int)(threadIdx.x & 1) : 0;
     const float lim2 = kSplitNear2 * sp.rate2;
-    load_rec_split(L + kRec * NP, C);
+    load_rec_split(L + kRec * np, C);
 #pragma unroll
     for (int c = 0; c < 3; ++c) C[c] = TPP == 2 && parity == 1 ? F2{0.0f, 0.0f} : f2_add(base[c], C[c]);
-    unsigned near = 0, mine = parity == 0 ? 1u << NP : 0u;
-#pragma unroll
-    for (int jj = (NP + TPP - 1) / TPP - 1; jj >= 0; --jj) {
+    unsigned near = 0, mine = parity == 0 ? 1u << np : 0u;
+#pragma unroll kUnroll
+    for (int jj = (np + TPP - 1) / TPP - 1; jj >= 0; --jj) {
         const int j = TPP * jj + parity;
-        if (j < NP) {
+        if (j < np) {
             F2 P[3];
             load_rec_split(L + kRec * j, P);
             if (!kick_split(X, P, sc.tg[j], sc.rc2[j], lim2, C)) near |= 1u << j;
@@ -146,7 +149,7 @@ __device__ __forceinline__ int kick_sum(double x, double y, double z, const F2 (
             for (int c = 0; c < 3; ++c) C[c] = base[c];
         }
         if (!act) near = 0;
-        if (TPP == 2 || near) hit = kick_near<NP>(near, x, y, z, L, pc, N);
+        if (TPP == 2 || near) hit = kick_near(near, np, x, y, z, L, pc, N);
         if constexpr (TPP == 2) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) N[c] += __shfl_xor_sync(kFullMask, N[c], 1);
@@ -180,14 +183,13 @@ static __device__ __noinline__ bool drift_fp64(const ParticleConsts& pc, bool pa
 }
 
 // Removal test without a kick (used at t_0).
-template <int NP>
-__device__ __forceinline__ int test_only(double x, double y, double z, const double* __restrict__ L,
+__device__ __forceinline__ int test_only(int np, double x, double y, double z, const double* __restrict__ L,
                                          const double (&rc2)[kMaxPlanets], double rmax2) {
     int hit = 0;
     const double r2 = fma(x, x, fma(y, y, z * z));
     if (__double_as_longlong(rmax2) != 0 && lt_nonneg(rmax2, r2)) hit = GLISSE_REMOVED_ESCAPE;
-#pragma unroll
-    for (int j = NP - 1; j >= 0; --j) {
+#pragma unroll 1
+    for (int j = np - 1; j >= 0; --j) {
         double px, py, pz;
         load_rec(L + kRec * j, px, py, pz);
         const double dx = x - px, dy = y - py, dz = z - pz;
@@ -222,11 +224,12 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
                                              const double* __restrict__ L, int64_t step0, int nsteps, bool test_first,
                                              double& x, double& y, double& z, double& vx, double& vy, double& vz,
                                              bool& act, int& reason, int64_t& rstep, bool open_in = false,
-                                             bool close_out = true, PublishTo pub = {}) {
-    const int S = log_stride(NP);
+                                             bool close_out = true, PublishTo pub = {}, int np_any = 0) {
+    const int np = NP >= 0 ? NP : np_any;
+    const int S = log_stride(np);
 
     if (test_first) {
-        const int h = test_only<NP>(x, y, z, L, pc.rc2, pc.rmax2);
+        const int h = test_only(np, x, y, z, L, pc.rc2, pc.rmax2);
         if (act && h != 0) {
             act = false;
             reason = h;
@@ -241,7 +244,7 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
         F2 C[3];
         double N[3];
         bool exact;
-        kick_sum<NP, TPP>(x, y, z, X, base, float_speed(r2, vx, vy, vz), act, L, pc, sc, C, N, exact);
+        kick_sum<NP, TPP>(np, x, y, z, X, base, float_speed(r2, vx, vy, vz), act, L, pc, sc, C, N, exact);
         if (act) {
             vx = fma(0.5, f2_sum(C[0]), vx);
             vy = fma(0.5, f2_sum(C[1]), vy);
@@ -335,7 +338,7 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
         F2 C[3];
         double N[3];
         bool exact;
-        const int enc = kick_sum<NP, TPP>(x, y, z, X, base, sp, act, Ln, pc, sc, C, N, exact);
+        const int enc = kick_sum<NP, TPP>(np, x, y, z, X, base, sp, act, Ln, pc, sc, C, N, exact);
         hit = enc ? enc : hit;
         const bool last = k + 1 == nsteps;
         if (last) {
@@ -457,39 +460,112 @@ __global__ void __launch_bounds__(kParticleBlock, GLISSE_PARTICLE_MIN_BLOCKS)
 // ---------------------------------------------------------------------------
 // Task mode: persistent warps over (group, sub-chunk) tasks.
 //
-// Every warp of a chunk does the same work, so with one thread per slot the
-// chunk lasts as long as the SM partition holding the most warps: at 6.06
-// warps per partition on average, the busiest has 7 and the pipe is 87%
-// used.  A particle's steps are serial, so balance needs smaller units of
-// work: the segment is cut into sub-chunks of sub_steps steps, and a task is
-// one group of 32 slots (the members of one warp of the plain launch) over
-// one sub-chunk.  Tasks are taken in order from a counter by a fixed number of
-// resident warps, so every partition keeps the same number of busy warps
-// until the last round of tasks.  Task (g, s) needs (g, s - 1) finished: it
-// is taken n_groups tasks later, by when the launch has that many warps'
-// worth of work behind it (the host uses task mode only when groups
-// outnumber resident warps by half again), and the warp waits, bounded, on
-// the group's counter of finished sub-chunks.  Sub-chunk cuts are open cuts,
-// so the result is bit-identical to the plain launch: same members per warp,
+// With one thread per slot a chunk lasts as long as the SM partition holding the
+// most warps, or the slowest ones (a group with a particle near a planet or a
+// pericentre takes longer).  A particle's steps are serial, so balance needs
+// smaller units of work: the segment is cut into sub-chunks of sub_steps steps, and
+// a task is one group of 32 slots (the members of one warp of the plain launch) over
+// one sub-chunk.  A fixed number of resident warps takes tasks: the first sub-chunk
+// of every group in order, then whichever group's previous sub-chunk finished
+// first (a queue: a finished task appends its group's next one).  With more groups
+// than resident warps a task is nearly always ready.  A group that has fallen behind
+// the others (one with a particle near a planet or a pericentre) is not put back:
+// its warp goes on with it, so that it does not finish last.  Sub-chunk cuts are
+// open cuts, so the result is bit-identical to the plain launch: same members per warp,
 // same steps, same kicks.
+//
+// A warp without a task waits, bounded, until its entry of the queue appears or every
+// group is finished.  The wait cannot deadlock: an unfinished group is either being
+// run (and its task ends in an append, in the next task or in the group's end) or in the
+// queue; if every running warp waited, all tickets before the first waiting one
+// would have been used up, the unfinished groups would be appended entries that no
+// ticket took, and the first waiting ticket is the next of those.
 // ---------------------------------------------------------------------------
 constexpr int kSubSteps = 32;
-// a wait for the previous sub-chunk of a group gives up after this many polls
-// (~64 ns each: seconds, where a sub-chunk takes a millisecond at most)
+constexpr int kMaxSub = 32;  // sub-chunks per segment at most (5 bits of a queue entry)
+// a wait for the queue gives up after this many polls (~64 ns each: seconds, where a
+// sub-chunk takes a millisecond at most)
 constexpr int kGroupWaitPolls = 1 << 25;
 
-__device__ __forceinline__ int ld_acquire(const int32_t* p) {
-    int v;
+__host__ __device__ inline int task_sub_steps(int nsteps) {
+    return max(kSubSteps, (nsteps + kMaxSub - 1) / kMaxSub);
+}
+
+__device__ __forceinline__ unsigned ld_acquire(const uint32_t* p) {
+    unsigned v;
     asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 
-__device__ __forceinline__ void st_release(int32_t* p, int v) {
+__device__ __forceinline__ void st_release(uint32_t* p, unsigned v) {
     asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// at most four blocks per SM (task_warps_per_partition), so up to 128 registers per thread
-constexpr int kTaskMaxBlocks = 4;
+// queue[0] counts the appends, queue[1] the finished groups; queue[2 + k] is the k-th append:
+// 1 + 32 group + sub-chunk.
+enum TaskState { kTaskReady, kTaskNone, kTaskTimeout };
+
+// The task of ticket t: group and sub-chunk (the same on the whole warp).
+__device__ __forceinline__ TaskState task_of_ticket(int64_t t, int64_t n_groups, const uint32_t* queue,
+                                                    int polls_limit, int64_t& g, int& s) {
+    if (t < n_groups) {
+        g = t;
+        s = 0;
+        return kTaskReady;
+    }
+    unsigned v = 0;
+    int state = kTaskReady;
+    if ((threadIdx.x & 31) == 0) {
+        const int limit = polls_limit > 0 ? polls_limit : kGroupWaitPolls;
+        const uint32_t* p = queue + 2 + (t - n_groups);
+        int polls = 0;
+        while ((v = ld_acquire(p)) == 0u) {
+            if ((int64_t)ld_acquire(queue + 1) >= n_groups) {
+                state = kTaskNone;
+                break;
+            }
+            if (++polls >= limit) {
+                state = kTaskTimeout;
+                break;
+            }
+            __nanosleep(64);
+        }
+    }
+    v = __shfl_sync(kFullMask, v, 0);
+    state = __shfl_sync(kFullMask, state, 0);
+    __syncwarp();
+    g = (int64_t)((v - 1u) >> 5);
+    s = (int)((v - 1u) & 31u);
+    return (TaskState)state;
+}
+
+// After task (g, s): publishes every lane's stores.  True when the warp is to go on with
+// (g, s + 1): the group is behind by more than half of the tasks that the queue holds
+// (warps: resident warps; taken: the ticket counter).  Else the group's next task goes
+// to the queue, or the group is finished.
+template <class Counter>
+__device__ __forceinline__ bool task_done(uint32_t* queue, const Counter* taken, int64_t g, int s, int n_sub,
+                                          int64_t n_groups, int64_t warps) {
+    __threadfence();
+    __syncwarp();
+    int on = 0;
+    if ((threadIdx.x & 31) == 0) {
+        if (s + 1 >= n_sub) {
+            if (n_sub > 1) atomicAdd(queue + 1, 1u);
+        } else {
+            const int64_t now = (int64_t)*reinterpret_cast<const volatile Counter*>(taken);
+            on = 2 * (now - (s * n_groups + g)) > n_groups + warps;
+            if (!on) {
+                const unsigned pos = atomicAdd(queue, 1u);
+                st_release(queue + 2 + pos, 1u + 32u * (unsigned)g + (unsigned)(s + 1));
+            }
+        }
+    }
+    return __shfl_sync(kFullMask, on, 0) != 0;
+}
+
+// at most five blocks per SM (task_warps_per_partition), so up to 96 registers per thread
+constexpr int kTaskMaxBlocks = 5;
 
 template <int NP>
 __global__ void __launch_bounds__(kParticleBlock, kTaskMaxBlocks)
@@ -505,71 +581,58 @@ __global__ void __launch_bounds__(kParticleBlock, kTaskMaxBlocks)
         if (lane == 0) t = atomicAdd(ta.task_counter, 1ull);
         t = __shfl_sync(kFullMask, t, 0);
         if ((int64_t)t >= n_tasks) break;
-        const int64_t g = (int64_t)t % ta.n_groups;
-        const int s = (int)((int64_t)t / ta.n_groups);
-        if (s > 0) {
-            int ok = 1;
-            if (lane == 0) {
-                const int limit = ta.wait_polls > 0 ? ta.wait_polls : kGroupWaitPolls;
-                int polls = 0;
-                while (ld_acquire(ta.group_done + g) < s && ++polls < limit) __nanosleep(64);
-                ok = polls < limit;
+        int64_t g;
+        int s;
+        const TaskState got = task_of_ticket((int64_t)t, ta.n_groups, ta.queue, ta.wait_polls, g, s);
+        if (got == kTaskTimeout && lane == 0) atomicExch(ta.status, GLISSE_E_TIMEOUT);
+        if (got != kTaskReady) break;
+        do {
+            const int64_t i = g * 32 + lane;
+            const bool in = i < a.n;
+            double x = 1.0, y = 0.0, z = 0.0, vx = 0.0, vy = 6.283185307179586, vz = 0.0;
+            bool act = false;
+            if (in) {
+                // written by another warp's task (L2 is coherent, this SM's L1 may not be)
+                x = __ldcg(a.st + i);
+                y = __ldcg(a.st + ld + i);
+                z = __ldcg(a.st + 2 * ld + i);
+                vx = __ldcg(a.st + 3 * ld + i);
+                vy = __ldcg(a.st + 4 * ld + i);
+                vz = __ldcg(a.st + 5 * ld + i);
+                act = __ldcg(a.alive + i) != 0;
             }
-            ok = __shfl_sync(kFullMask, ok, 0);
-            if (!ok) {
-                if (lane == 0) atomicExch(ta.status, GLISSE_E_TIMEOUT);
-                break;
+            const bool started = act;
+            int reason = 0;
+            int64_t rstep = -1;
+            const int k0 = s * ta.sub_steps;
+            const int m = min(ta.sub_steps, a.nsteps - k0);
+            const bool last = s + 1 == n_sub;
+            advance_lane<NP, kDriftConverge, 1, true>(pc, sc, a.log + (size_t)k0 * S, a.step0 + k0, m,
+                                                      a.test_first != 0 && s == 0, x, y, z, vx, vy, vz, act, reason,
+                                                      rstep, s > 0 || a.open_in != 0, last ? a.close_out != 0 : false,
+                                                      PublishTo{a.id, last ? a.out_state : nullptr, i});
+            if (a.steps_done) {
+                const unsigned adv = !started ? 0u : (rstep >= 0 ? (unsigned)(rstep - (a.step0 + k0)) : (unsigned)m);
+                const unsigned wsum = __reduce_add_sync(kFullMask, adv);
+                if (lane == 0 && wsum) atomicAdd(a.steps_done, (unsigned long long)wsum);
             }
-        }
-        __syncwarp();
-        const int64_t i = g * 32 + lane;
-        const bool in = i < a.n;
-        double x = 1.0, y = 0.0, z = 0.0, vx = 0.0, vy = 6.283185307179586, vz = 0.0;
-        bool act = false;
-        if (in) {
-            // written by another warp's task (L2 is coherent, this SM's L1 may not be)
-            x = __ldcg(a.st + i);
-            y = __ldcg(a.st + ld + i);
-            z = __ldcg(a.st + 2 * ld + i);
-            vx = __ldcg(a.st + 3 * ld + i);
-            vy = __ldcg(a.st + 4 * ld + i);
-            vz = __ldcg(a.st + 5 * ld + i);
-            act = __ldcg(a.alive + i) != 0;
-        }
-        const bool started = act;
-        int reason = 0;
-        int64_t rstep = -1;
-        const int k0 = s * ta.sub_steps;
-        const int m = min(ta.sub_steps, a.nsteps - k0);
-        const bool last = s + 1 == n_sub;
-        advance_lane<NP, kDriftConverge, 1, true>(pc, sc, a.log + (size_t)k0 * S, a.step0 + k0, m,
-                                                  a.test_first != 0 && s == 0, x, y, z, vx, vy, vz, act, reason,
-                                                  rstep, s > 0 || a.open_in != 0, last ? a.close_out != 0 : false,
-                                                  PublishTo{a.id, last ? a.out_state : nullptr, i});
-        if (a.steps_done) {
-            const unsigned adv = !started ? 0u : (rstep >= 0 ? (unsigned)(rstep - (a.step0 + k0)) : (unsigned)m);
-            const unsigned wsum = __reduce_add_sync(kFullMask, adv);
-            if (lane == 0 && wsum) atomicAdd(a.steps_done, (unsigned long long)wsum);
-        }
-        if (last && a.live_out) {
-            const unsigned wl = __reduce_add_sync(kFullMask, act ? 1u : 0u);
-            if (lane == 0 && wl) atomicAdd(a.live_out, (unsigned long long)wl);
-        }
-        if (in) {
-            __stcg(a.st + i, x);
-            __stcg(a.st + ld + i, y);
-            __stcg(a.st + 2 * ld + i, z);
-            __stcg(a.st + 3 * ld + i, vx);
-            __stcg(a.st + 4 * ld + i, vy);
-            __stcg(a.st + 5 * ld + i, vz);
-            __stcg(a.alive + i, (uint8_t)(act ? 1 : 0));
-            if (rstep >= 0) store_removed(a.id[i], x, y, z, vx, vy, vz, rstep, reason, a.out_state, a.out_step,
-                                          a.out_reason);
-        }
-        // every lane's stores before the group's counter moves on (release at device scope)
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) st_release(ta.group_done + g, s + 1);
+            if (last && a.live_out) {
+                const unsigned wl = __reduce_add_sync(kFullMask, act ? 1u : 0u);
+                if (lane == 0 && wl) atomicAdd(a.live_out, (unsigned long long)wl);
+            }
+            if (in) {
+                __stcg(a.st + i, x);
+                __stcg(a.st + ld + i, y);
+                __stcg(a.st + 2 * ld + i, z);
+                __stcg(a.st + 3 * ld + i, vx);
+                __stcg(a.st + 4 * ld + i, vy);
+                __stcg(a.st + 5 * ld + i, vz);
+                __stcg(a.alive + i, (uint8_t)(act ? 1 : 0));
+                if (rstep >= 0) store_removed(a.id[i], x, y, z, vx, vy, vz, rstep, reason, a.out_state, a.out_step,
+                                              a.out_reason);
+            }
+        } while (task_done(ta.queue, ta.task_counter, g, s++, n_sub, ta.n_groups,
+                           (int64_t)gridDim.x * (kParticleBlock / 32)));
     }
 }
 
@@ -590,19 +653,25 @@ inline cudaError_t particle_smem_cap(const void* kernel, int64_t grid, size_t* s
     return residency_cap_smem(kernel, per_sm, GLISSE_PARTICLE_MIN_BLOCKS, smem);
 }
 
-// Warps per SM partition for task mode, or 0 for the plain launch: task mode
-// pays when the groups outnumber the resident warps by half again (waits are
-// then rare) with at least two busy warps per partition (one warp alone keeps
-// the FP64 pipe ~70% busy); at most four (enough to saturate it).
+// Warps per SM partition for task mode, or 0 for the plain launch.  Few warps leave the
+// FP64 pipe idle between a warp's dependent instructions; many make a group's
+// sub-chunks slower, and with it the tail in which the last groups finish.  Milliseconds
+// per 1024 steps at 2 | 3 | 4 | 5 warps (8 bodies, particles at 2-46 au, groups per partition in
+// brackets; plain launch in front):
+//     32768 [1.7]   2.8: 2.9 | 3.1 | 3.5 | 4.8        65536 [3.4]   4.5: 4.3 | 4.0 | 4.3 | 4.5
+//     98304 [5.1]   6.9: 6.3 | 5.3 | 5.4 | 5.6       131072 [6.7]   7.5: 8.3 | 7.0 | 6.6 | 6.9
+//    262144 [13.5] 12.6: 15.7 | 12.7 | 11.8 | 11.3
+// (the last row 5 bodies).  A launch without a quarter more groups than warps is the plain one: its
+// groups would never wait for a warp, and one thread per slot needs no tickets.
 inline int task_warps_per_partition(int64_t n, int nsteps, int n_sm) {
     const int64_t groups = (n + 31) / 32;
     const int64_t partitions = 4 * (int64_t)std::max(n_sm - 1, 1);
     if (nsteps < 2 * kSubSteps) return 0;
-    const int64_t k = (2 * groups) / (3 * partitions);
-    return k >= 2 ? (int)std::min<int64_t>(k, kTaskMaxBlocks) : 0;
+    const int64_t k = std::min<int64_t>(2 + groups / (3 * partitions), kTaskMaxBlocks);
+    return 4 * groups >= 5 * k * partitions ? (int)k : 0;
 }
 
-// tb: the task-mode buffers (counter, per-group counters, status), or null for the plain launch.
+// tb: the task-mode buffers (counter, queue, status), or null for the plain launch.
 // force_tasks: task mode whatever the size (two warps per partition at least; GLISSE_LAUNCH_TASKS).
 template <int MODE>
 cudaError_t launch_particle_chunk_mode(int np, const ChunkArgs& a, const ParticleConsts& pc, cudaStream_t s,
@@ -620,10 +689,12 @@ cudaError_t launch_particle_chunk_mode(int np, const ChunkArgs& a, const Particl
         if (tb && force_tasks && k == 0) k = 2;
         if (k > 0) {
             TaskArgs b = *tb;
-            b.sub_steps = kSubSteps;
+            b.sub_steps = task_sub_steps(a.nsteps);
             b.n_groups = (int32_t)((a.n + 31) / 32);
             e = cudaMemsetAsync(b.task_counter, 0, sizeof(unsigned long long), s);
-            if (e == cudaSuccess) e = cudaMemsetAsync(b.group_done, 0, sizeof(int32_t) * (size_t)b.n_groups, s);
+            const size_t n_sub = (size_t)((a.nsteps + b.sub_steps - 1) / b.sub_steps);
+            if (e == cudaSuccess)
+                e = cudaMemsetAsync(b.queue, 0, sizeof(uint32_t) * (2 + (size_t)b.n_groups * (n_sub - 1)), s);
             if (e != cudaSuccess) return e;
             // k blocks of four warps per SM, one SM's worth short (the ephemeris holds one)
             const int64_t grid = (int64_t)k * std::max(nsm - 1, 1);
@@ -633,7 +704,7 @@ cudaError_t launch_particle_chunk_mode(int np, const ChunkArgs& a, const Particl
     case N:                                                                                              \
         e = particle_smem_cap(reinterpret_cast<const void*>(particle_tasks_kernel<N>), grid, &smem);     \
         if (e != cudaSuccess) return e;                                                                  \
-        particle_tasks_kernel<N><<<(unsigned)grid, kParticleBlock, smem, s>>>(a, pc, sc, b);                 \
+        particle_tasks_kernel<N><<<(unsigned)grid, kParticleBlock, smem, s>>>(a, pc, sc, b);             \
         break;
                 GLISSE_TCASE(0)
                 GLISSE_TCASE(1)
@@ -658,7 +729,7 @@ cudaError_t launch_particle_chunk_mode(int np, const ChunkArgs& a, const Particl
     case N:                                                                                               \
         e = particle_smem_cap(reinterpret_cast<const void*>(particle_chunk_kernel<N, MODE>), grid, &smem); \
         if (e != cudaSuccess) return e;                                                                   \
-        particle_chunk_kernel<N, MODE><<<(unsigned)grid, kParticleBlock, smem, s>>>(a, pc, sc);              \
+        particle_chunk_kernel<N, MODE><<<(unsigned)grid, kParticleBlock, smem, s>>>(a, pc, sc);           \
         break;
         GLISSE_CASE(0)
         GLISSE_CASE(1)

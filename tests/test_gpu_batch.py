@@ -132,6 +132,24 @@ def test_batch_equals_single_system_runs(G, chunk):
         assert e.max() <= parity.state_tol(n), (s, e.max())
 
 
+@pytest.mark.parametrize("steps", [33, 64, 97])
+def test_sub_chunk_tasks_are_bit_identical(G, steps):
+    """With a quarter more 32-particle groups than resident warps the particle kernel runs
+    sub-chunks of 32 steps from a queue, else whole chunks.  3200 systems of 1 to 40
+    particles take the queue (two to four sub-chunks, whole and ragged), two halves of
+    them do not: the same systems give the same bits, removals included."""
+    b = gi.make_batched(seed=21, n_systems=3200, n_min=1, n_max=40)
+    po, ao = offsets(b)
+    whole = run_batch(G, b, steps, chunk_steps=128)
+    for lo, hi in ((0, 1600), (1600, 3200)):
+        rows = slice(ao[lo], ao[hi])
+        half = run_batch(G, {"star_mass": b["star_mass"][lo:hi], "n_planets": b["n_planets"][lo:hi],
+                             "planets": b["planets"][po[lo]:po[hi]], "n_particles": b["n_particles"][lo:hi],
+                             "particles": b["particles"][rows], "dt": b["dt"][lo:hi]}, steps, chunk_steps=128)
+        for k in ("state", "alive", "removal_step", "removal_reason"):
+            np.testing.assert_array_equal(half[k], whole[k][rows], err_msg=k)
+
+
 def test_graph_replay_equals_direct_launches(G):
     b = small_batch(n_systems=5, seed=9)
     g1 = run_batch(G, b, 900, splits=[300, 300, 300], chunk_steps=256)  # captured chunk graphs
