@@ -715,7 +715,7 @@ class DiffMap:
 
     checkpoint_every: K >= 1 stores the state every K steps and recomputes each
     segment in the backward pass; 0 (tape) records every step in the forward
-    pass ((112 + 16 N_p) B per particle-step) so the backward pass is the reverse
+    pass (112 B per particle-step) so the backward pass is the reverse
     sweep alone (about half the cost); GLISSE_DIFF_AUTO takes the tape when it
     fits in half of the free device memory.  The reverse sweep for the growth
     indicator's gradient needs checkpoints, or GLISSE_DIFF_TAPE_TANGENT: a tape

@@ -16,17 +16,24 @@
 // kick of dt (their Jacobians, tau A(r) at the same r, merge the same way);
 // at a segment boundary and at the end they stay half kicks.  Backward: for each K-step segment from
 // the last, the thread recomputes the segment from its checkpoint, keeping the
-// pre-drift state, the post-drift position, the solved universal anomaly s,
-// the reduced time tau, G_4, G_5 and 1/R of every step in a scratch buffer,
-// then runs the adjoint kicks and drifts backwards through it (the other
-// G-functions follow from G_4, G_5 by their recurrence: no second solve and no
-// second series).
-// Tape mode (checkpoint_every = 0) keeps that record for every step of the
-// run, written by the forward pass itself: the backward pass is the reverse
-// sweep alone, at 112 + 16 N_p B per particle-step of device memory (176 B with
-// four planets: 115 GB for 65536 particles over 10^4 steps, which HBM holds).
-// The record also keeps the closing kick's s_j and 1/|d_j|^2, so the sweep
-// does not evaluate the kick's reciprocals again.
+// pre-drift state and the post-drift position of every step in a scratch buffer,
+// then runs the adjoint kicks and drifts backwards through it.  Tape mode
+// (checkpoint_every = 0) keeps that record for every step of the run, written by
+// the forward pass itself: the backward pass is the reverse sweep alone, at 112 B
+// per particle-step of device memory (73 GB for 65536 particles over 10^4
+// steps, which HBM holds).
+//
+// The state takes the particle map's step, FP64 sums and float pairs for the
+// corrections to them (split_step.cuh), and so do tangents and cotangents
+// (split_diff.cuh): FP64 instructions bound all of these kernels when everything was FP64
+// (151 per forward step, 173 per reverse step with four planets; 32768 particles, 512 steps:
+// 6.1 and 6.3 ms).  Now 25 and ~45: 1.7 and 3.1 ms, bound by the latency of the dependent
+// float operations at two warps per SM partition (4096 particles take 1.6 and 2.7 ms).
+// Drifts outside the pairs' domain and planets that are near take FP64, per lane; the
+// record keeps such a drift's s, tau, G_4, G_5 and 1/R, so the sweep neither solves
+// for them nor sums their series again.  The pairs' scalars it forms again
+// (reading 88 B a step is dearer than ~350 float operations).
+//
 // A removed particle's output is its frozen state; its derivatives are those
 // of that frozen state (the steps after removal contribute nothing).
 //
@@ -47,6 +54,8 @@
 #include "glisse_internal.h"
 #include "nvtx_range.h"
 #include "drift_diff.cuh"
+#include "particle_map.cuh"
+#include "split_diff.cuh"
 
 namespace glisse {
 cudaError_t launch_eph_setup(const double*, int, double, double, int, double, PlanetConsts*, double*, int*,
@@ -55,23 +64,22 @@ cudaError_t launch_eph_chunk(const PlanetConsts*, double*, double, int, double*,
                              int* progress = nullptr, const int* stop = nullptr);
 
 constexpr int kMaxTangents = 6;
-constexpr int kScratchRows = 14;  // pre-drift state (6), post-drift position (3), s, tau, G_4, G_5, 1/R
-// Rows of one step's record: the kScratchRows of the drift, then the closing kick's
-// s_j = tau G m_j / |d_j|^3 and 1/|d_j|^2 (40-bit) for each planet j, which the forward
-// pass (or the recompute) forms anyway, so the reverse sweep reads them instead of
-// evaluating two reciprocals per planet again.
-__host__ __device__ constexpr int record_rows(int np) { return kScratchRows + 2 * np; }
+// Rows of one step's record: pre-drift state (6), post-drift position (3), then s, tau, G_4,
+// G_5, 1/R where the drift was solved in FP64; s = 0 where it was not (float pairs: its
+// scalars cost the reverse sweep less to form again than to read).
+constexpr int kScratchRows = 14;
 constexpr int kDiffBlock = 128;
 
 struct DiffArgs {
+    int32_t np;             // planets (at run time: one code per kernel)
     const double* log;      // [nsteps + 1] planet log steps
     int64_t n;              // particles
     int64_t nsteps;
     int32_t K;              // checkpoint interval
     int32_t ntan;           // tangent vectors (0..kMaxTangents)
     int32_t tape;           // 1: scratch holds every step, written by the forward pass
-    int32_t rec_rows;       // rows of one step's record in scratch: record_rows(NP), or
-                            // record_rows(NP) + 9 when the tape also keeps tangent 0
+    int32_t rec_rows;       // rows of one step's record in scratch: kScratchRows, or
+                            // kScratchRows + 9 when the tape also keeps tangent 0
     int32_t tan_row;        // first of tangent 0's 9 rows in a record (0: not kept)
     const double* state0;   // [n][6]
     double* state1;         // [n][6]
@@ -91,30 +99,143 @@ struct DiffArgs {
     double* gradt0;         // [n][6] out: gradient with respect to t0
 };
 
-// v += tau a(r) for the log step L; returns the lowest planet index whose encounter test fires.
-// rec (optional): a step record (stride ld), which receives s_j and 1/|d_j|^2 of this kick.
-template <int NP>
-__device__ __forceinline__ int kick_state(double st[6], const double* __restrict__ L, double tau,
-                                          const double (&tgm)[kMaxPlanets], const double (&rc2)[kMaxPlanets],
-                                          double* rec = nullptr, int64_t ld = 0) {
-    const double h0x = L[kRec * NP], h0y = L[kRec * NP + 1], h0z = L[kRec * NP + 2];
-    st[3] = fma(tau, h0x, st[3]);
-    st[4] = fma(tau, h0y, st[4]);
-    st[5] = fma(tau, h0z, st[5]);
-    int hit = 0;
+// ---------------------------------------------------------------------------
+// One step's state, the same arithmetic wherever a kernel forms it (forward pass,
+// recompute, growth): the particle map's, FP64 sums and float pairs (split_step.cuh),
+// with drift_scalars for the lanes outside the pairs' domain.  All per lane: a
+// step does not depend on the other lanes of its warp.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void split_position(const double (&st)[6], F2 (&X)[3], double& r2) {
 #pragma unroll
-    for (int j = NP - 1; j >= 0; --j) {
-        const double dx = st[0] - L[kRec * j], dy = st[1] - L[kRec * j + 1], dz = st[2] - L[kRec * j + 2];
-        const double d2 = fma(dx, dx, fma(dy, dy, dz * dz));
-        hit = lt_nonneg(d2, rc2[j]) ? (j + 1) : hit;
-        const double s = k_rcube(d2, tgm[j]);
-        if (rec) {
-            rec[(kScratchRows + j) * ld] = s;
-            rec[(kScratchRows + NP + j) * ld] = rcp_40(d2);
+    for (int c = 0; c < 3; ++c) X[c] = f2_split(st[c]);
+    r2 = fma(st[0], st[0], fma(st[1], st[1], st[2] * st[2]));
+}
+
+// v += (dt / 2) a(r) at the log step L: the opening half kick of a segment.
+__device__ __forceinline__ void kick_open(int np, double (&st)[6], const F2 (&X)[3], double r2, const double* __restrict__ L,
+                                          const ParticleConsts& pc, const SplitConsts& sc) {
+    constexpr F2 kZero = {0.0f, 0.0f};
+    const F2 base[3] = {kZero, kZero, kZero};
+    F2 C[3];
+    double N[3];
+    bool exact;
+    kick_sum<kAnyNp, 1, false>(np, st[0], st[1], st[2], X, base, float_speed(r2, st[3], st[4], st[5]), true, L, pc, sc, C,
+                           N, exact);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        st[3 + c] = fma(0.5, f2_sum(C[c]), st[3 + c]);
+        if (exact) st[3 + c] = fma(0.5, N[c], st[3 + c]);
+    }
+}
+
+// The FP64 drift of one lane: pre -> st and tangents t[T][6]; rec (or null): the step's record.
+static __device__ __noinline__ bool drift64(const ParticleConsts& pc, const double* pre, double* st, int T, double* t,
+                                            double* rec, int64_t ld) {
+    double x[6];
+    for (int c = 0; c < 6; ++c) x[c] = pre[c];
+    DriftScalars d;
+    if (!drift_scalars(pc.mu, pc.dt, x, d)) return false;
+    for (int c = 0; c < 3; ++c) {
+        st[c] = fma(d.f, x[c], d.g * x[3 + c]);
+        st[3 + c] = fma(d.fd, x[c], d.gd * x[3 + c]);
+    }
+    if (rec) {
+        rec[9 * ld] = d.s;
+        rec[10 * ld] = d.tau;
+        rec[11 * ld] = d.G[4];
+        rec[12 * ld] = d.G[5];
+        rec[13 * ld] = d.inv_R;
+    }
+    for (int q = 0; q < T; ++q) {
+        double w[6];
+        for (int c = 0; c < 6; ++c) w[c] = t[6 * q + c];
+        drift_tangent(pc.mu, x, d, w);
+        for (int c = 0; c < 6; ++c) t[6 * q + c] = w[c];
+    }
+    return true;
+}
+
+// Drift of a step: pre (position split: X, r2) -> n, the velocity without base (the part
+// still in pairs); t: T tangents; rec: the step's record or null (stride ld).  Returns 0, or
+// the removal reason of a failed step (t unchanged).
+template <int T, int TA>
+__device__ __forceinline__ int diff_drift(const ParticleConsts& pc, const SplitConsts& sc, const double (&pre)[6],
+                                          const F2 (&X)[3], double r2, double (&n)[6], F2 (&base)[3], Speed& sp,
+                                          double (&t)[TA][6], double* rec, int64_t ld) {
+    const F2 V[3] = {f2_split(pre[3]), f2_split(pre[4]), f2_split(pre[5])};
+    DriftFactors f;
+    DriftSeries ser;
+    const bool pairs =
+        drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp, T > 0 ? &ser : nullptr) && in_float_range(r2);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        base[c] = f2_mul(f.gdm1, V[c]);
+        n[c] = fma(f.fm1, pre[c], fma(f.g, pre[3 + c], pre[c]));
+        n[3 + c] = fma(f.fd, pre[c], pre[3 + c]);
+    }
+    if (pairs && rec) rec[9 * ld] = 0.0;
+    if (!pairs) {
+        double x[6], w[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) x[c] = pre[c];
+        if (!drift64(pc, x, w, 0, nullptr, rec, ld)) return GLISSE_REMOVED_KEPLER;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) n[c] = w[c];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) base[c] = F2{0.0f, 0.0f};
+    }
+    bool bad = false;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) bad |= nonfinite_bits(n[c]);
+    if (bad) return GLISSE_REMOVED_NONFINITE;
+    if constexpr (T > 0) {
+        DriftJac J;
+        drift_jac(ser, J);
+#pragma unroll
+        for (int q = 0; q < T; ++q) {
+            int e;
+            if (scale_exponent(t[q], e) && pairs) {
+                drift_tangent_split(sc.dt, ser, f, J, pre, X, V, t[q], e);
+            } else {
+                double x[6], w[6], u[6];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    x[c] = pre[c];
+                    u[c] = t[q][c];
+                }
+                drift64(pc, x, w, 1, u, nullptr, 0);
+#pragma unroll
+                for (int c = 0; c < 6; ++c) t[q][c] = u[c];
+            }
         }
-        st[3] = fma(-s, dx, st[3]);
-        st[4] = fma(-s, dy, st[4]);
-        st[5] = fma(-s, dz, st[5]);
+    }
+    return 0;
+}
+
+// The tests at t_{k+1} and the closing kick at the log step L, of dt (merge) or dt / 2, in place.
+// n, base: diff_drift's; X, r2: those of n.  Returns the removal reason or 0; a removed
+// particle keeps the drifted state.
+__device__ __forceinline__ int kick_close(int np, double (&n)[6], const F2 (&base)[3], Speed sp, const F2 (&X)[3], double r2,
+                                          bool merge, const double* __restrict__ L, const ParticleConsts& pc,
+                                          const SplitConsts& sc) {
+    int hit = (__double_as_longlong(pc.rmax2) != 0 && lt_nonneg(pc.rmax2, r2)) ? GLISSE_REMOVED_ESCAPE : 0;
+    if (!in_float_range(r2)) sp.v2 = -1.0f;
+    F2 C[3];
+    double N[3];
+    bool exact;
+    const int enc = kick_sum<kAnyNp, 1, false>(np, n[0], n[1], n[2], X, base, sp, true, L, pc, sc, C, N, exact);
+    hit = enc ? enc : hit;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (hit) {
+            n[3 + c] += f2_sum(base[c]);
+        } else if (merge) {
+            n[3 + c] += f2_sum(C[c]);
+            if (exact) n[3 + c] += N[c];
+        } else {
+            n[3 + c] = fma(0.5, f2_sum(f2_add(base[c], C[c])), n[3 + c]);
+            if (exact) n[3 + c] = fma(0.5, N[c], n[3 + c]);
+        }
     }
     return hit;
 }
@@ -125,12 +246,11 @@ __device__ __forceinline__ int kick_state(double st[6], const double* __restrict
 // ~tau G m_j / |d|^3 (1e-4 or less) of the step's Jacobian.
 // Generic over the scalar type: with ad::Dual components (r, dr) and (w, dw) it
 // also gives d(tau A(r) w) = tau A(r) dw + tau (dA(r)[dr]) w.
-// Planets in kick_state's order (last first), as kick_tangents sums them.
-template <int NP, class T>
-__device__ __forceinline__ void kick_jac(const T r[3], const double* __restrict__ L,
+template <class T>
+__device__ __forceinline__ void kick_jac(int np, const T r[3], const double* __restrict__ L,
                                          const double (&tgm)[kMaxPlanets], const T w[3], T out[3]) {
-#pragma unroll
-    for (int j = NP - 1; j >= 0; --j) {
+#pragma unroll 4
+    for (int j = np - 1; j >= 0; --j) {
         const T dx = r[0] - L[kRec * j], dy = r[1] - L[kRec * j + 1], dz = r[2] - L[kRec * j + 2];
         const T d2 = fma(dx, dx, fma(dy, dy, dz * dz));
         const T s = k_rcube(d2, tgm[j]);
@@ -141,57 +261,57 @@ __device__ __forceinline__ void kick_jac(const T r[3], const double* __restrict_
     }
 }
 
-// kick_state and the tangent's kick_jac in one pass over the planets, sharing the
-// separation, |d|^2 and s_j: the velocity v and the tangent's velocity part tv get
-// exactly what kick_state and kick_jac give them (same expressions, same order);
-// w is the tangent's position part.  Returns what kick_state returns.
-template <int NP>
-__device__ __forceinline__ int kick_tangent(const double r[3], double v[3], const double w[3], double tv[3],
-                                            const double* __restrict__ L, double tau,
-                                            const double (&tgm)[kMaxPlanets], const double (&rc2)[kMaxPlanets],
-                                            double* rec = nullptr, int64_t ld = 0) {
-    const double h0x = L[kRec * NP], h0y = L[kRec * NP + 1], h0z = L[kRec * NP + 2];
-    v[0] = fma(tau, h0x, v[0]);
-    v[1] = fma(tau, h0y, v[1]);
-    v[2] = fma(tau, h0z, v[2]);
-    int hit = 0;
+// out += tau A(r) w at the log step L, tau = dt or (half) dt / 2, w the velocity or position part of a
+// cotangent or tangent whose scale is e (ok: scale_exponent's): planets in pairs
+// (kick_jac_split), in FP64 those the particle is near to, by the rate (mu / r^3)^(1/2).
+__device__ __forceinline__ void kick_jac_add(int np, const double r[3], const F2 (&X)[3], const double* __restrict__ L,
+                                             const ParticleConsts& pc, const SplitConsts& sc, bool half, bool ok,
+                                             int e, const double w[3], double out[3]) {
+    const int h = max(max(exp_bits(r[0]), exp_bits(r[1])), exp_bits(r[2]));
+    const float y = rsqrt_f32(fmaf(X[0].h, X[0].h, fmaf(X[1].h, X[1].h, X[2].h * X[2].h)));
+    const float lim2 = (unsigned)(h - (1023 - 49)) <= 98u && ok ? kSplitNear2 * (d2f_bits(pc.mu) * y * y * y) : -1.0f;
+    const double tau = half ? 0.5 : 1.0;
+    F2 W[3], acc[3];
 #pragma unroll
-    for (int j = NP - 1; j >= 0; --j) {
-        const double dx = r[0] - L[kRec * j], dy = r[1] - L[kRec * j + 1], dz = r[2] - L[kRec * j + 2];
-        const double d2 = fma(dx, dx, fma(dy, dy, dz * dz));
-        hit = lt_nonneg(d2, rc2[j]) ? (j + 1) : hit;
-        const double s = k_rcube(d2, tgm[j]);
-        const double inv = rcp_40(d2);
-        if (rec) {
-            rec[(kScratchRows + j) * ld] = s;
-            rec[(kScratchRows + NP + j) * ld] = inv;
-        }
-        v[0] = fma(-s, dx, v[0]);
-        v[1] = fma(-s, dy, v[1]);
-        v[2] = fma(-s, dz, v[2]);
-        const double c = (3.0 * fma(dx, w[0], fma(dy, w[1], dz * w[2]))) * inv;
-        tv[0] = fma(-s, fma(-c, dx, w[0]), tv[0]);
-        tv[1] = fma(-s, fma(-c, dy, w[1]), tv[1]);
-        tv[2] = fma(-s, fma(-c, dz, w[2]), tv[2]);
+    for (int c = 0; c < 3; ++c) {
+        W[c] = f2_split_scaled(w[c], ok ? e : 0);
+        acc[c] = F2{0.0f, 0.0f};
     }
-    return hit;
+    unsigned near = 0;
+#pragma unroll 4
+    for (int j = np - 1; j >= 0; --j) {
+        F2 P[3];
+        load_rec_split(L + kRec * j, P);
+        if (!kick_jac_split(X, P, sc.tg[j], lim2, W, acc)) near |= 1u << j;
+    }
+    double N[3] = {0.0, 0.0, 0.0};
+    if (near) {
+#pragma unroll 1
+        for (int j = np - 1; j >= 0; --j) {
+            if (!((near >> j) & 1u)) continue;
+            const double dx = r[0] - L[kRec * j], dy = r[1] - L[kRec * j + 1], dz = r[2] - L[kRec * j + 2];
+            const double d2 = fma(dx, dx, fma(dy, dy, dz * dz));
+            const double s = k_rcube(d2, pc.tgm_full[j]);
+            const double c = (3.0 * fma(dx, w[0], fma(dy, w[1], dz * w[2]))) * rcp_full(d2);
+            N[0] = fma(-s, fma(-c, dx, w[0]), N[0]);
+            N[1] = fma(-s, fma(-c, dy, w[1]), N[1]);
+            N[2] = fma(-s, fma(-c, dz, w[2]), N[2]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        out[c] = fma(tau, f2_double_scaled(acc[c], ok ? e : 0), out[c]);
+        if (near) out[c] = fma(tau, N[c], out[c]);
+    }
 }
 
-// kick_jac at the closing kick of a recorded step: s_j and 1/|d_j|^2 come from the
-// record (rec: its kick rows, stride ld), the same values kick_jac would form.
-template <int NP>
-__device__ __forceinline__ void kick_jac_rec(const double r[3], const double* __restrict__ L,
-                                             const double* __restrict__ rec, int64_t ld, const double w[3],
-                                             double out[3]) {
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-        const double dx = r[0] - L[kRec * j], dy = r[1] - L[kRec * j + 1], dz = r[2] - L[kRec * j + 2];
-        const double s = rec[j * ld];
-        const double c = (3.0 * fma(dx, w[0], fma(dy, w[1], dz * w[2]))) * rec[(NP + j) * ld];
-        out[0] = fma(-s, fma(-c, dx, w[0]), out[0]);
-        out[1] = fma(-s, fma(-c, dy, w[1]), out[1]);
-        out[2] = fma(-s, fma(-c, dz, w[2]), out[2]);
-    }
+// The same for a whole tangent t: dv += tau A(r) dr.
+__device__ __forceinline__ void kick_jac_tangent(int np, const double r[3], const F2 (&X)[3], const double* __restrict__ L,
+                                                 const ParticleConsts& pc, const SplitConsts& sc, bool half,
+                                                 double (&t)[6]) {
+    int e;
+    const bool ok = scale_exponent(t, e);
+    kick_jac_add(np, r, X, L, pc, sc, half, ok, e, t, t + 3);
 }
 
 // Steps [k_lo, k_hi) of the forward pass for particle i (stopping at a removal): state
@@ -199,119 +319,80 @@ __device__ __forceinline__ void kick_jac_rec(const double r[3], const double* __
 // into the previous closing kick).  Checkpoints at every multiple of K and the tape
 // record of each step are written as the steps pass, so any split of [0, nsteps) into
 // consecutive calls does the same arithmetic.
-template <int NP, int T, int TA>
-__device__ __forceinline__ void forward_steps(const DiffArgs& a, const ParticleConsts& pc, int64_t i, double (&st)[6],
-                                              double (&t)[TA][6], int64_t& rstep, int& reason, bool& opened,
-                                              int64_t k_lo, int64_t k_hi) {
-    const int S = log_stride(NP);
-    const bool has_rmax = __double_as_longlong(pc.rmax) != 0;
+template <int T, int TA>
+__device__ __forceinline__ void forward_steps(const DiffArgs& a, const ParticleConsts& pc, const SplitConsts& sc,
+                                              int64_t i, double (&st)[6], double (&t)[TA][6], int64_t& rstep,
+                                              int& reason, bool& opened, int64_t k_lo, int64_t k_hi) {
+    const int np = a.np, S = log_stride(np);
+    F2 X[3];
+    double r2;
+    split_position(st, X, r2);
+    // place of step k in its checkpoint segment (a 64-bit division per step is as long as a planet's kick)
+    int in_seg = (int)(k_lo % a.K);
     for (int64_t k = k_lo; k < k_hi && rstep < 0; ++k) {
-        if (k % a.K == 0) {
-            double* cp = a.ckpt + (k / a.K) * 6 * a.n;
+        if (in_seg == 0) {
+            const int64_t seg = k / a.K;
+            double* cp = a.ckpt + seg * 6 * a.n;
             for (int c = 0; c < 6; ++c) cp[c * a.n + i] = st[c];
             if (T > 0 && a.ckpt_t) {
-                double* ct = a.ckpt_t + (k / a.K) * 6 * a.n;
+                double* ct = a.ckpt_t + seg * 6 * a.n;
                 for (int c = 0; c < 6; ++c) ct[c * a.n + i] = t[0][c];
             }
         }
+        if (++in_seg == a.K) in_seg = 0;
         const double* L0 = a.log + k * S;
         const double* L1 = L0 + S;
         // opening half kick (A is evaluated at r, which the kick leaves unchanged)
         if (!opened) {
-            if constexpr (T == 1) {
-                kick_tangent<NP>(st, st + 3, t[0], t[0] + 3, L0, pc.half_dt, pc.tgm_half, pc.rc2);
-            } else {
 #pragma unroll
-                for (int q = 0; q < T; ++q) kick_jac<NP>(st, L0, pc.tgm_half, t[q], t[q] + 3);
-                kick_state<NP>(st, L0, pc.half_dt, pc.tgm_half, pc.rc2);
-            }
+            for (int q = 0; q < T; ++q) kick_jac_tangent(np, st, X, L0, pc, sc, true, t[q]);
+            kick_open(np, st, X, r2, L0, pc, sc);
         }
-        double pre[6];
-        for (int c = 0; c < 6; ++c) pre[c] = st[c];
         double* tp = a.tape ? a.scratch + k * a.rec_rows * a.n + i : nullptr;
         if (tp)
-            for (int c = 0; c < 6; ++c) tp[c * a.n] = pre[c];
+            for (int c = 0; c < 6; ++c) tp[c * a.n] = st[c];
         // the tape of the growth gradient's sweep also keeps tangent 0 (before the drift)
         if constexpr (T >= 1)
             if (tp && a.tan_row > 0)
                 for (int c = 0; c < 6; ++c) tp[(a.tan_row + c) * a.n] = t[0][c];
-        DriftScalars d;
-        if (!drift_scalars(pc.mu, pc.dt, pre, d)) {
+        double n[6];
+        F2 base[3];
+        Speed sp;
+        const int failed = diff_drift<T, TA>(pc, sc, st, X, r2, n, base, sp, t, tp, a.n);
+        if (failed) {
             rstep = k + 1;
-            reason = GLISSE_REMOVED_KEPLER;
+            reason = failed;
             break;
         }
-        for (int c = 0; c < 3; ++c) {
-            st[c] = fma(d.f, pre[c], d.g * pre[3 + c]);
-            st[3 + c] = fma(d.fd, pre[c], d.gd * pre[3 + c]);
-        }
-        if (tp) {
+        for (int c = 0; c < 6; ++c) st[c] = n[c];
+        if (tp)
             for (int c = 0; c < 3; ++c) tp[(6 + c) * a.n] = st[c];
-            tp[9 * a.n] = d.s;
-            tp[10 * a.n] = d.tau;
-            tp[11 * a.n] = d.G[4];
-            tp[12 * a.n] = d.G[5];
-            tp[13 * a.n] = d.inv_R;
-        }
-        bool bad = false;
-        for (int c = 0; c < 6; ++c) bad |= nonfinite_bits(st[c]);
-        if (bad) {
-            for (int c = 0; c < 6; ++c) st[c] = pre[c];
-            rstep = k + 1;
-            reason = GLISSE_REMOVED_NONFINITE;
-            break;
-        }
-#pragma unroll
-        for (int q = 0; q < T; ++q) drift_tangent(pc.mu, pre, d, t[q]);
         if constexpr (T >= 1)
             if (tp && a.tan_row > 0)
                 for (int c = 0; c < 3; ++c) tp[(a.tan_row + 6 + c) * a.n] = t[0][c];
         // tests at t_{k+1}, then the closing kick (merged with the next opening one
         // inside a segment)
-        const bool merge = (k + 1 < a.nsteps) && ((k + 1) % a.K != 0);
-        const double tau = merge ? pc.dt : pc.half_dt;
-        const double(&tgm)[kMaxPlanets] = merge ? pc.tgm_full : pc.tgm_half;
-        const double r2 = fma(st[0], st[0], fma(st[1], st[1], st[2] * st[2]));
-        int hit = (has_rmax && lt_nonneg(pc.rmax2, r2)) ? GLISSE_REMOVED_ESCAPE : 0;
-        double nst[6], ntv[3];
-        for (int c = 0; c < 6; ++c) nst[c] = st[c];
-        int enc;
-        if constexpr (T == 1) {
-            for (int c = 0; c < 3; ++c) ntv[c] = t[0][3 + c];
-            enc = kick_tangent<NP>(st, nst + 3, t[0], ntv, L1, tau, tgm, pc.rc2, tp, a.n);
-        } else {
-            enc = kick_state<NP>(nst, L1, tau, tgm, pc.rc2, tp, a.n);
-        }
-        hit = enc ? enc : hit;
+        const bool merge = (k + 1 < a.nsteps) && in_seg != 0;
+        split_position(st, X, r2);
+        const int hit = kick_close(np, st, base, sp, X, r2, merge, L1, pc, sc);
         if (hit) {
             rstep = k + 1;
             reason = hit;
             break;
         }
-        if constexpr (T == 1) {
-            for (int c = 0; c < 3; ++c) t[0][3 + c] = ntv[c];
-        } else {
 #pragma unroll
-            for (int q = 0; q < T; ++q) kick_jac<NP>(st, L1, tgm, t[q], t[q] + 3);
-        }
-        for (int c = 0; c < 6; ++c) st[c] = nst[c];
+        for (int q = 0; q < T; ++q) kick_jac_tangent(np, st, X, L1, pc, sc, !merge, t[q]);
         opened = merge;
     }
 }
 
 // The removal test at t_0 (before the first step).
-template <int NP>
 __device__ __forceinline__ void forward_test_first(const DiffArgs& a, const ParticleConsts& pc, const double (&st)[6],
                                                    int64_t& rstep, int& reason) {
-    const bool has_rmax = __double_as_longlong(pc.rmax) != 0;
-    double tmp[6];
-    for (int c = 0; c < 6; ++c) tmp[c] = st[c];
-    const int hit = kick_state<NP>(tmp, a.log, 0.0, pc.tgm_half, pc.rc2);
-    const double r2 = fma(st[0], st[0], fma(st[1], st[1], st[2] * st[2]));
-    const int esc = (has_rmax && lt_nonneg(pc.rmax2, r2)) ? GLISSE_REMOVED_ESCAPE : 0;
-    if (hit || esc) {
+    const int hit = test_only(a.np, st[0], st[1], st[2], a.log, pc.rc2, pc.rmax2);
+    if (hit) {
         rstep = 0;
-        reason = hit ? hit : esc;
+        reason = hit;
     }
 }
 
@@ -325,8 +406,8 @@ __device__ __forceinline__ double norm2(const double (&t)[TA][6]) {
 
 // TMAX: compile-time tangent capacity (0, 1 or kMaxTangents) so that the
 // tangent vectors stay in registers; tangents a.ntan..TMAX-1 are zero.
-template <int NP, int TMAX>
-__global__ void __launch_bounds__(kDiffBlock, TMAX == 0 ? 7 : (TMAX == 1 ? 4 : 1)) diff_forward_kernel(const DiffArgs a, const ParticleConsts pc) {
+template <int TMAX>
+__global__ void __launch_bounds__(kDiffBlock, TMAX <= 1 ? 4 : 1) diff_forward_kernel(const DiffArgs a, const __grid_constant__ ParticleConsts pc, const __grid_constant__ SplitConsts sc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     constexpr int T = TMAX;
@@ -340,9 +421,9 @@ __global__ void __launch_bounds__(kDiffBlock, TMAX == 0 ? 7 : (TMAX == 1 ? 4 : 1
     const double n0 = norm2<TA>(t);
     int64_t rstep = -1;
     int reason = 0;
-    forward_test_first<NP>(a, pc, st, rstep, reason);
+    forward_test_first(a, pc, st, rstep, reason);
     bool opened = false;
-    forward_steps<NP, T, TA>(a, pc, i, st, t, rstep, reason, opened, 0, a.nsteps);
+    forward_steps<T, TA>(a, pc, sc, i, st, t, rstep, reason, opened, 0, a.nsteps);
     for (int c = 0; c < 6; ++c) a.state1[6 * i + c] = st[c];
 #pragma unroll
     for (int q = 0; q < T; ++q)
@@ -363,87 +444,75 @@ __global__ void __launch_bounds__(kDiffBlock, TMAX == 0 ? 7 : (TMAX == 1 ? 4 : 1
 // dt = d(J t0)/dx0 [e_c], through the same steps, kick merging and removals as
 // the forward pass.  Then dg/dx0_c = (J t0) . dt / |J t0|^2.
 // a.grad0[6 i + c] <- dg/dx0_c; a.log_growth[i] <- g (from the c = 0 thread).
-template <int NP>
-__global__ void __launch_bounds__(kDiffBlock) diff_growth_kernel(const DiffArgs a, const ParticleConsts pc) {
+__global__ void __launch_bounds__(kDiffBlock) diff_growth_kernel(const DiffArgs a, const __grid_constant__ ParticleConsts pc,
+        const __grid_constant__ SplitConsts sc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int c = blockIdx.y;
     if (i >= a.n) return;
-    const int S = log_stride(NP);
-    double st[6], dx[6];
+    const int np = a.np, S = log_stride(np);
+    double st[6], dx[6], tv[1][6];  // tv: the forward pass's tangent, bit for bit, as t's value
     Dual t[6];
     for (int k = 0; k < 6; ++k) {
         st[k] = a.state0[6 * i + k];
         dx[k] = (k == c) ? 1.0 : 0.0;
         t[k] = {a.tan0[6 * i + k], 0.0};
+        tv[0][k] = t[k].v;
     }
     double n0 = 0.0;
     for (int k = 0; k < 6; ++k) n0 = fma(t[k].v, t[k].v, n0);
-    bool removed = false;
-    const bool has_rmax = __double_as_longlong(pc.rmax) != 0;
-    {
-        double tmp[6];
-        for (int k = 0; k < 6; ++k) tmp[k] = st[k];
-        const int hit = kick_state<NP>(tmp, a.log, 0.0, pc.tgm_half, pc.rc2);
-        const double r2 = fma(st[0], st[0], fma(st[1], st[1], st[2] * st[2]));
-        removed = hit != 0 || (has_rmax && lt_nonneg(pc.rmax2, r2));
-    }
+    int64_t rstep = -1;
+    int reason = 0;
+    forward_test_first(a, pc, st, rstep, reason);
+    bool removed = rstep >= 0;
     bool opened = false;
+    F2 X[3];
+    double r2;
+    split_position(st, X, r2);
     for (int64_t k = 0; k < a.nsteps && !removed; ++k) {
         const double* L0 = a.log + k * S;
         const double* L1 = L0 + S;
         if (!opened) {
             const Dual rd[3] = {{st[0], dx[0]}, {st[1], dx[1]}, {st[2], dx[2]}};
-            kick_jac<NP>(rd, L0, pc.tgm_half, t, t + 3);
-            kick_jac<NP>(st, L0, pc.tgm_half, dx, dx + 3);
-            kick_state<NP>(st, L0, pc.half_dt, pc.tgm_half, pc.rc2);
+            kick_jac(np, rd, L0, pc.tgm_half, t, t + 3);
+            kick_jac(np, st, L0, pc.tgm_half, dx, dx + 3);
+            kick_jac_tangent(np, st, X, L0, pc, sc, true, tv[0]);
+            kick_open(np, st, X, r2, L0, pc, sc);
         }
-        double pre[6], pdx[6];
+        double pdx[6], n[6];
         for (int q = 0; q < 6; ++q) {
-            pre[q] = st[q];
             pdx[q] = dx[q];
+            t[q].v = tv[0][q];
         }
+        F2 base[3];
+        Speed sp;
         DriftScalars d;
-        if (!drift_scalars(pc.mu, pc.dt, pre, d)) {
-            removed = true;
+        if (diff_drift<1, 1>(pc, sc, st, X, r2, n, base, sp, tv, nullptr, 0) ||
+            !drift_scalars(pc.mu, pc.dt, st, d))
             break;
-        }
-        for (int q = 0; q < 3; ++q) {
-            st[q] = fma(d.f, pre[q], d.g * pre[3 + q]);
-            st[3 + q] = fma(d.fd, pre[q], d.gd * pre[3 + q]);
-        }
-        bool bad = false;
-        for (int q = 0; q < 6; ++q) bad |= nonfinite_bits(st[q]);
-        if (bad) {
-            for (int q = 0; q < 6; ++q) st[q] = pre[q];
-            removed = true;
-            break;
-        }
-        drift_tangent(pc.mu, pre, d, dx);
+        drift_tangent(pc.mu, st, d, dx);
         {
-            const DriftScalarsT<Dual> e = drift_lift(pc.mu, pre, pdx, d);
+            const DriftScalarsT<Dual> e = drift_lift(pc.mu, st, pdx, d);
             Dual pd[6];
-            for (int q = 0; q < 6; ++q) pd[q] = {pre[q], pdx[q]};
+            for (int q = 0; q < 6; ++q) pd[q] = {st[q], pdx[q]};
             drift_tangent(pc.mu, pd, e, t);
         }
-        const bool merge = (k + 1 < a.nsteps) && ((k + 1) % a.K != 0);
-        const double tau = merge ? pc.dt : pc.half_dt;
-        const double(&tgm)[kMaxPlanets] = merge ? pc.tgm_full : pc.tgm_half;
-        const double r2 = fma(st[0], st[0], fma(st[1], st[1], st[2] * st[2]));
-        double nst[6];
-        for (int q = 0; q < 6; ++q) nst[q] = st[q];
-        const int enc = kick_state<NP>(nst, L1, tau, tgm, pc.rc2);
-        if (enc != 0 || (has_rmax && lt_nonneg(pc.rmax2, r2))) {
-            removed = true;
-            break;
+        for (int q = 0; q < 6; ++q) {
+            st[q] = n[q];
+            t[q].v = tv[0][q];
         }
+        const bool merge = (k + 1 < a.nsteps) && ((k + 1) % a.K != 0);
+        const double(&tgm)[kMaxPlanets] = merge ? pc.tgm_full : pc.tgm_half;
+        split_position(st, X, r2);
+        if (kick_close(np, st, base, sp, X, r2, merge, L1, pc, sc)) break;
         const Dual rd[3] = {{st[0], dx[0]}, {st[1], dx[1]}, {st[2], dx[2]}};
-        kick_jac<NP>(rd, L1, tgm, t, t + 3);
-        kick_jac<NP>(st, L1, tgm, dx, dx + 3);
-        for (int q = 0; q < 6; ++q) st[q] = nst[q];
+        kick_jac(np, rd, L1, tgm, t, t + 3);
+        kick_jac(np, st, L1, tgm, dx, dx + 3);
+        kick_jac_tangent(np, st, X, L1, pc, sc, !merge, tv[0]);
         opened = merge;
     }
     double n1 = 0.0, p1 = 0.0;
     for (int k = 0; k < 6; ++k) {
+        t[k].v = tv[0][k];
         n1 = fma(t[k].v, t[k].v, n1);
         p1 = fma(t[k].v, t[k].d, p1);
     }
@@ -457,75 +526,119 @@ __global__ void __launch_bounds__(kDiffBlock) diff_growth_kernel(const DiffArgs 
 // steps [s_lo, s_hi) of the segment, last step first.  l: cotangent of the state at s_hi
 // in, at s_lo out.  The plain launch sweeps whole segments; the task launch cuts the one
 // segment of tape mode into sub-chunks.
-template <int NP>
-__device__ __forceinline__ void backward_piece(const DiffArgs& a, const ParticleConsts& pc, int64_t i,
-                                               double (&l)[6], int64_t cseg, int64_t k0, int64_t k1,
+__device__ __forceinline__ void prefetch_l1(const double* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
+// The FP64 drift adjoint of one lane; rec5: s, tau, G_4, G_5, 1/R, or s = 0 to solve for them.
+static __device__ __noinline__ void adjoint64(const ParticleConsts& pc, const double* pre, const double* rec5,
+                                              double* l) {
+    double x[6], w[6];
+    for (int c = 0; c < 6; ++c) {
+        x[c] = pre[c];
+        w[c] = l[c];
+    }
+    DriftScalars d;
+    if (rec5[0] == 0.0) {
+        drift_scalars(pc.mu, pc.dt, x, d);
+    } else {
+        drift_restore(pc.mu, pc.dt, x, rec5[0], rec5[1], d);
+        drift_finish_stored(pc.mu, d, rec5[2], rec5[3], rec5[4]);
+    }
+    drift_adjoint(pc.mu, x, d, w);
+    for (int c = 0; c < 6; ++c) l[c] = w[c];
+}
+
+__device__ __forceinline__ void backward_piece(const DiffArgs& a, const ParticleConsts& pc, const SplitConsts& sc,
+                                               int64_t i, double (&l)[6], int64_t cseg, int64_t k0, int64_t k1,
                                                int64_t s_lo, int64_t s_hi, int64_t kend, bool cut_after_drift,
                                                bool cut_before_drift) {
-    const int S = log_stride(NP);
-    double st[6];
-    const double* cp = a.ckpt + cseg * 6 * a.n;
-    for (int c = 0; c < 6; ++c) st[c] = cp[c * a.n + i];
+    const int np = a.np, S = log_stride(np);
     // recompute the segment: pre-drift state (6) and post-drift position (3) per step
     // (in tape mode the forward pass wrote them already)
-    const int64_t krec = a.tape ? k0 : k1;  // steps to recompute: none in tape mode
-    for (int64_t k = k0; k < krec; ++k) {
-        const double* L0 = a.log + k * S;
-        if (k == k0) kick_state<NP>(st, L0, pc.half_dt, pc.tgm_half, pc.rc2);  // else merged below
-        double* sc = a.scratch + (k - k0) * a.rec_rows * a.n + i;
-        for (int c = 0; c < 6; ++c) sc[c * a.n] = st[c];
-        if (k == kend - 1 && cut_before_drift) break;
-        DriftScalars d;
-        drift_scalars(pc.mu, pc.dt, st, d);
-        sc[9 * a.n] = d.s;
-        sc[10 * a.n] = d.tau;
-        sc[11 * a.n] = d.G[4];
-        sc[12 * a.n] = d.G[5];
-        sc[13 * a.n] = d.inv_R;
-        double pre[6];
-        for (int c = 0; c < 6; ++c) pre[c] = st[c];
-        for (int c = 0; c < 3; ++c) {
-            st[c] = fma(d.f, pre[c], d.g * pre[3 + c]);
-            st[3 + c] = fma(d.fd, pre[c], d.gd * pre[3 + c]);
-        }
-        for (int c = 0; c < 3; ++c) sc[(6 + c) * a.n] = st[c];
-        // closing kick of step k merged with the opening kick of step k + 1 (as in the forward
-        // pass); at the segment's end the closing half kick, recorded only
-        if (k + 1 < krec) {
-            kick_state<NP>(st, a.log + (k + 1) * S, pc.dt, pc.tgm_full, pc.rc2, sc, a.n);
-        } else {
-            double tmp[6];
-            for (int c = 0; c < 6; ++c) tmp[c] = st[c];
-            kick_state<NP>(tmp, a.log + (k + 1) * S, pc.half_dt, pc.tgm_half, pc.rc2, sc, a.n);
+    if (!a.tape) {
+        double st[6];
+        const double* cp = a.ckpt + cseg * 6 * a.n;
+        for (int c = 0; c < 6; ++c) st[c] = cp[c * a.n + i];
+        F2 X[3];
+        double r2;
+        split_position(st, X, r2);
+        kick_open(np, st, X, r2, a.log + k0 * S, pc, sc);
+        for (int64_t k = k0; k < k1; ++k) {
+            double* rec = a.scratch + (k - k0) * a.rec_rows * a.n + i;
+            for (int c = 0; c < 6; ++c) rec[c * a.n] = st[c];
+            if (k == kend - 1 && cut_before_drift) break;
+            double n[6], none[1][6];
+            F2 base[3];
+            Speed sp;
+            diff_drift<0, 1>(pc, sc, st, X, r2, n, base, sp, none, rec, a.n);
+            for (int c = 0; c < 6; ++c) st[c] = n[c];
+            for (int c = 0; c < 3; ++c) rec[(6 + c) * a.n] = st[c];
+            // closing kick of step k merged with the opening kick of step k + 1 (as in the forward
+            // pass); the one at the segment's end is not needed
+            if (k + 1 == k1) break;
+            split_position(st, X, r2);
+            kick_close(np, st, base, sp, X, r2, true, a.log + (k + 1) * S, pc, sc);
         }
     }
     // adjoint sweep, last step first
     for (int64_t k = s_hi - 1; k >= s_lo; --k) {
-        const double* sc = a.scratch + (k - k0) * a.rec_rows * a.n + i;
-        double pre[6], post[3];
-        for (int c = 0; c < 6; ++c) pre[c] = sc[c * a.n];
-        for (int c = 0; c < 3; ++c) post[c] = sc[(6 + c) * a.n];
+        const double* rec = a.scratch + (k - k0) * a.rec_rows * a.n + i;
+        double pre[6];
+        for (int c = 0; c < 6; ++c) pre[c] = rec[c * a.n];
+        const double s = rec[9 * a.n];
+        // the record of step k - 1 on its way while step k is computed
+        if (k > s_lo) {
+#pragma unroll
+            for (int c = 0; c < 10; ++c) prefetch_l1(rec + c * a.n - (int64_t)a.rec_rows * a.n);
+        }
         const bool last = (k == kend - 1);
         if (!(last && (cut_after_drift || cut_before_drift))) {
             // closing kick at t_{k+1}: lr += tau A(post) lv, tau = dt inside the segment
-            // (merged with the opening kick of step k + 1), dt/2 at its end; its s_j and
-            // 1/|d_j|^2 are in the step's record
-            kick_jac_rec<NP>(post, a.log + (k + 1) * S, sc + kScratchRows * a.n, a.n, l + 3, l);
+            // (merged with the opening kick of step k + 1), dt/2 at its end
+            double post[3];
+            for (int c = 0; c < 3; ++c) post[c] = rec[(6 + c) * a.n];
+            const F2 Y[3] = {f2_split(post[0]), f2_split(post[1]), f2_split(post[2])};
+            int e;
+            const bool ok = scale_exponent(l, e);
+            kick_jac_add(np, post, Y, a.log + (k + 1) * S, pc, sc, k + 1 == k1, ok, e, l + 3, l);
         }
+        F2 X[3];
+        double r2;
+        split_position(pre, X, r2);
         if (!(last && cut_before_drift)) {
-            DriftScalars d;
-            drift_restore(pc.mu, pc.dt, pre, sc[9 * a.n], sc[10 * a.n], d);
-            drift_finish_stored(pc.mu, d, sc[11 * a.n], sc[12 * a.n], sc[13 * a.n]);
-            drift_adjoint(pc.mu, pre, d, l);
+            int e;
+            if (scale_exponent(l, e) && s == 0.0) {
+                const F2 V[3] = {f2_split(pre[3]), f2_split(pre[4]), f2_split(pre[5])};
+                DriftFactors f;
+                DriftSeries ser;
+                DriftJac J;
+                Speed sp;
+                drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp, &ser);
+                drift_jac(ser, J);
+                drift_adjoint_split(sc.dt, ser, f, J, pre, X, V, l, e);
+            } else {
+                double x[6], w[6], r5[5] = {s, 0.0, 0.0, 0.0, 0.0};
+                if (s != 0.0)
+                    for (int c = 1; c < 5; ++c) r5[c] = rec[(9 + c) * a.n];
+                for (int c = 0; c < 6; ++c) {
+                    x[c] = pre[c];
+                    w[c] = l[c];
+                }
+                adjoint64(pc, x, r5, w);
+                for (int c = 0; c < 6; ++c) l[c] = w[c];
+            }
         }
         // opening half kick at t_k (only at the segment start; inside, it is part of
         // the previous step's merged closing kick): lr += (dt/2) A(pre) lv
-        if (k == k0) kick_jac<NP>(pre, a.log + k * S, pc.tgm_half, l + 3, l);
+        if (k == k0) {
+            int e;
+            const bool ok = scale_exponent(l, e);
+            kick_jac_add(np, pre, X, a.log + k * S, pc, sc, true, ok, e, l + 3, l);
+        }
     }
 }
 
-template <int NP>
-__global__ void __launch_bounds__(kDiffBlock, 4) diff_backward_kernel(const DiffArgs a, const ParticleConsts pc) {
+__global__ void __launch_bounds__(kDiffBlock, 4) diff_backward_kernel(const DiffArgs a, const __grid_constant__ ParticleConsts pc,
+        const __grid_constant__ SplitConsts sc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     double l[6];
@@ -542,7 +655,7 @@ __global__ void __launch_bounds__(kDiffBlock, 4) diff_backward_kernel(const Diff
         for (int64_t cseg = nseg - 1; cseg >= 0; --cseg) {
             const int64_t k0 = cseg * a.K;
             const int64_t k1 = min(k0 + (int64_t)a.K, kend);
-            backward_piece<NP>(a, pc, i, l, cseg, k0, k1, k0, k1, kend, cut_after_drift, cut_before_drift);
+            backward_piece(a, pc, sc, i, l, cseg, k0, k1, k0, k1, kend, cut_after_drift, cut_before_drift);
         }
     }
     for (int c = 0; c < 6; ++c) a.grad0[6 * i + c] = l[c];
@@ -579,9 +692,8 @@ __device__ __forceinline__ void diff_st_release(int32_t* p, int v) {
     asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <int NP>
-__global__ void __launch_bounds__(kDiffBlock, 4) diff_backward_tasks_kernel(const DiffArgs a, const ParticleConsts pc,
-                                                                            const DiffTaskArgs ta) {
+__global__ void __launch_bounds__(kDiffBlock, 4) diff_backward_tasks_kernel(const DiffArgs a, const __grid_constant__ ParticleConsts pc,
+        const __grid_constant__ SplitConsts sc, const DiffTaskArgs ta) {
     const int lane = threadIdx.x & 31;
     const int64_t n_tasks = (int64_t)ta.n_groups * ta.n_sub;
     for (;;) {
@@ -623,9 +735,9 @@ __global__ void __launch_bounds__(kDiffBlock, 4) diff_backward_tasks_kernel(cons
             const int64_t hi = min(lo + ta.sub, kend);
             if (hi > lo) {
                 if (a.tape)
-                    backward_piece<NP>(a, pc, i, l, 0, 0, kend, lo, hi, kend, cut_after_drift, cut_before_drift);
+                    backward_piece(a, pc, sc, i, l, 0, 0, kend, lo, hi, kend, cut_after_drift, cut_before_drift);
                 else
-                    backward_piece<NP>(a, pc, i, l, c_idx, lo, hi, lo, hi, kend, cut_after_drift, cut_before_drift);
+                    backward_piece(a, pc, sc, i, l, c_idx, lo, hi, lo, hi, kend, cut_after_drift, cut_before_drift);
             }
             for (int c = 0; c < 6; ++c) __stcg(a.grad0 + 6 * i + c, l[c]);
         }
@@ -643,9 +755,9 @@ __global__ void __launch_bounds__(kDiffBlock, 4) diff_backward_tasks_kernel(cons
 // pass.  The arithmetic is forward_steps', so the outputs equal the plain launch's bit for bit.
 constexpr int kFwdSub = 64;
 
-template <int NP, int TMAX>
-__global__ void __launch_bounds__(kDiffBlock, 4) diff_forward_tasks_kernel(const DiffArgs a, const ParticleConsts pc,
-                                                                           const DiffTaskArgs ta) {
+template <int TMAX>
+__global__ void __launch_bounds__(kDiffBlock, 4) diff_forward_tasks_kernel(const DiffArgs a, const __grid_constant__ ParticleConsts pc,
+        const __grid_constant__ SplitConsts sc, const DiffTaskArgs ta) {
     constexpr int T = TMAX;
     constexpr int TA = TMAX > 0 ? TMAX : 1;
     const int lane = threadIdx.x & 31;
@@ -684,7 +796,7 @@ __global__ void __launch_bounds__(kDiffBlock, 4) diff_forward_tasks_kernel(const
 #pragma unroll
                     for (int c = 0; c < 6; ++c) t[q][c] = (q < a.ntan) ? a.tan0[((int64_t)q * a.n + i) * 6 + c] : 0.0;
                 if (a.log_growth) a.log_growth[i] = norm2<TA>(t);  // |t0|^2, until the last task
-                forward_test_first<NP>(a, pc, st, rstep, reason);
+                forward_test_first(a, pc, st, rstep, reason);
             } else {
                 for (int c = 0; c < 6; ++c) st[c] = __ldcg(a.state1 + 6 * i + c);
 #pragma unroll
@@ -699,7 +811,7 @@ __global__ void __launch_bounds__(kDiffBlock, 4) diff_forward_tasks_kernel(const
             const int64_t hi = min(lo + ta.sub, a.nsteps);
             // inside a checkpoint segment the previous step's closing kick opened this one
             bool opened = lo > 0 && lo < a.nsteps && lo % a.K != 0;
-            forward_steps<NP, T, TA>(a, pc, i, st, t, rstep, reason, opened, lo, hi);
+            forward_steps<T, TA>(a, pc, sc, i, st, t, rstep, reason, opened, lo, hi);
             for (int c = 0; c < 6; ++c) __stcg(a.state1 + 6 * i + c, st[c]);
 #pragma unroll
             for (int q = 0; q < T; ++q)
@@ -733,11 +845,11 @@ constexpr int kScratchRowsG = kScratchRows + 9;
 // GLISSE_DIFF_TAPE_TANGENT, read from the forward call's record of every step.
 // a.grad0 <- lx at t_0 (= J^T grad_state1 + grad_growth dg/dstate0 at fixed t0);
 // a.gradt0 <- lt at t_0 minus grad_growth t0 / |t0|^2 (= dg/dt0 times grad_growth).
-template <int NP>
-__global__ void __launch_bounds__(kDiffBlock, 2) diff_backward_growth_kernel(const DiffArgs a, const ParticleConsts pc) {
+__global__ void __launch_bounds__(kDiffBlock, 2) diff_backward_growth_kernel(const DiffArgs a, const __grid_constant__ ParticleConsts pc,
+        const __grid_constant__ SplitConsts sc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
-    const int S = log_stride(NP);
+    const int np = a.np, S = log_stride(np);
     const double gg = a.gradg ? a.gradg[i] : 0.0;
     double nn = 0.0;
     for (int c = 0; c < 6; ++c) nn = fma(a.tanN[6 * i + c], a.tanN[6 * i + c], nn);
@@ -758,69 +870,69 @@ __global__ void __launch_bounds__(kDiffBlock, 2) diff_backward_growth_kernel(con
             const int64_t k0 = cseg * a.K;
             const int64_t k1 = min(k0 + (int64_t)a.K, kend);
             const int64_t krec = a.tape ? k0 : k1;  // steps to recompute: none with a tape
-            double st[6], t[6];
+            double st[6], t[1][6];
             const double* cp = a.ckpt + cseg * 6 * a.n;
             const double* ct = a.ckpt_t + cseg * 6 * a.n;
             for (int c = 0; c < 6; ++c) {
                 st[c] = cp[c * a.n + i];
-                t[c] = ct[c * a.n + i];
+                t[0][c] = ct[c * a.n + i];
             }
+            F2 X[3];
+            double r2;
+            split_position(st, X, r2);
             for (int64_t k = k0; k < krec; ++k) {
                 const double* L0 = a.log + k * S;
                 if (k == k0) {
-                    kick_jac<NP>(st, L0, pc.tgm_half, t, t + 3);
-                    kick_state<NP>(st, L0, pc.half_dt, pc.tgm_half, pc.rc2);
+                    kick_jac_tangent(np, st, X, L0, pc, sc, true, t[0]);
+                    kick_open(np, st, X, r2, L0, pc, sc);
                 }
-                double* sc = a.scratch + (k - k0) * rows * a.n + i;
+                double* rec = a.scratch + (k - k0) * rows * a.n + i;
                 for (int c = 0; c < 6; ++c) {
-                    sc[c * a.n] = st[c];
-                    sc[(trow + c) * a.n] = t[c];
+                    rec[c * a.n] = st[c];
+                    rec[(trow + c) * a.n] = t[0][c];
                 }
                 if (k == kend - 1 && cut_before_drift) break;
-                DriftScalars d;
-                drift_scalars(pc.mu, pc.dt, st, d);
-                sc[9 * a.n] = d.s;
-                sc[10 * a.n] = d.tau;
-                sc[11 * a.n] = d.G[4];
-                sc[12 * a.n] = d.G[5];
-                sc[13 * a.n] = d.inv_R;
-                double pre[6];
-                for (int c = 0; c < 6; ++c) pre[c] = st[c];
+                double n[6];
+                F2 base[3];
+                Speed sp;
+                diff_drift<1, 1>(pc, sc, st, X, r2, n, base, sp, t, rec, a.n);
+                for (int c = 0; c < 6; ++c) st[c] = n[c];
                 for (int c = 0; c < 3; ++c) {
-                    st[c] = fma(d.f, pre[c], d.g * pre[3 + c]);
-                    st[3 + c] = fma(d.fd, pre[c], d.gd * pre[3 + c]);
-                }
-                drift_tangent(pc.mu, pre, d, t);
-                for (int c = 0; c < 3; ++c) {
-                    sc[(6 + c) * a.n] = st[c];
-                    sc[(trow + 6 + c) * a.n] = t[c];
+                    rec[(6 + c) * a.n] = st[c];
+                    rec[(trow + 6 + c) * a.n] = t[0][c];
                 }
                 if (k + 1 < k1) {
-                    kick_jac<NP>(st, a.log + (k + 1) * S, pc.tgm_full, t, t + 3);
-                    kick_state<NP>(st, a.log + (k + 1) * S, pc.dt, pc.tgm_full, pc.rc2);
+                    split_position(st, X, r2);
+                    kick_close(np, st, base, sp, X, r2, true, a.log + (k + 1) * S, pc, sc);
+                    kick_jac_tangent(np, st, X, a.log + (k + 1) * S, pc, sc, false, t[0]);
                 }
             }
             for (int64_t k = k1 - 1; k >= k0; --k) {
-                const double* sc = a.scratch + (k - k0) * rows * a.n + i;
+                const double* rec = a.scratch + (k - k0) * rows * a.n + i;
                 double pre[6];
                 Dual pd[6], qd[3];
                 for (int c = 0; c < 6; ++c) {
-                    pre[c] = sc[c * a.n];
-                    pd[c] = {pre[c], sc[(trow + c) * a.n]};
+                    pre[c] = rec[c * a.n];
+                    pd[c] = {pre[c], rec[(trow + c) * a.n]};
                 }
-                for (int c = 0; c < 3; ++c) qd[c] = {sc[(6 + c) * a.n], sc[(trow + 6 + c) * a.n]};
+                for (int c = 0; c < 3; ++c) qd[c] = {rec[(6 + c) * a.n], rec[(trow + 6 + c) * a.n]};
                 const bool last = (k == kend - 1);
                 if (!(last && (cut_after_drift || cut_before_drift)))
-                    kick_jac<NP>(qd, a.log + (k + 1) * S, (k + 1 < k1) ? pc.tgm_full : pc.tgm_half, l + 3, l);
+                    kick_jac(np, qd, a.log + (k + 1) * S, (k + 1 < k1) ? pc.tgm_full : pc.tgm_half, l + 3, l);
                 if (!(last && cut_before_drift)) {
                     DriftScalars d;
-                    drift_restore(pc.mu, pc.dt, pre, sc[9 * a.n], sc[10 * a.n], d);
-                    drift_finish_stored(pc.mu, d, sc[11 * a.n], sc[12 * a.n], sc[13 * a.n]);
+                    const double s = rec[9 * a.n];
+                    if (s == 0.0) {
+                        drift_scalars(pc.mu, pc.dt, pre, d);
+                    } else {
+                        drift_restore(pc.mu, pc.dt, pre, s, rec[10 * a.n], d);
+                        drift_finish_stored(pc.mu, d, rec[11 * a.n], rec[12 * a.n], rec[13 * a.n]);
+                    }
                     const double tp[6] = {pd[0].d, pd[1].d, pd[2].d, pd[3].d, pd[4].d, pd[5].d};
                     const DriftScalarsT<Dual> e = drift_lift(pc.mu, pre, tp, d);
                     drift_adjoint(pc.mu, pd, e, l);
                 }
-                if (k == k0) kick_jac<NP>(pd, a.log + k * S, pc.tgm_half, l + 3, l);
+                if (k == k0) kick_jac(np, pd, a.log + k * S, pc.tgm_half, l + 3, l);
             }
         }
     }
@@ -836,38 +948,17 @@ __global__ void __launch_bounds__(kDiffBlock, 2) diff_backward_growth_kernel(con
     }
 }
 
-#define GLISSE_DIFF_SWITCH(KERNEL)                                         \
-    switch (np) {                                                          \
-        case 0: KERNEL<0><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        case 1: KERNEL<1><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        case 2: KERNEL<2><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        case 3: KERNEL<3><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        case 4: KERNEL<4><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        case 5: KERNEL<5><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        case 6: KERNEL<6><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        case 7: KERNEL<7><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        case 8: KERNEL<8><<<grid, kDiffBlock, 0, s>>>(a, pc); break;       \
-        default: return cudaErrorInvalidValue;                             \
-    }
+static SplitConsts split_consts(const ParticleConsts& pc) {
+    SplitConsts sc{};
+    split_step_consts(pc, sc);
+    for (int j = 0; j < kMaxPlanets; ++j) split_planet(pc, j, sc);
+    return sc;
+}
 
 template <int TMAX>
-static cudaError_t launch_diff_forward_t(int np, const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s) {
+static cudaError_t launch_diff_forward_t(const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s) {
     const unsigned grid = (unsigned)((a.n + kDiffBlock - 1) / kDiffBlock);
-    switch (np) {
-#define GLISSE_FWD_CASE(N) \
-    case N: diff_forward_kernel<N, TMAX><<<grid, kDiffBlock, 0, s>>>(a, pc); break;
-        GLISSE_FWD_CASE(0)
-        GLISSE_FWD_CASE(1)
-        GLISSE_FWD_CASE(2)
-        GLISSE_FWD_CASE(3)
-        GLISSE_FWD_CASE(4)
-        GLISSE_FWD_CASE(5)
-        GLISSE_FWD_CASE(6)
-        GLISSE_FWD_CASE(7)
-        GLISSE_FWD_CASE(8)
-#undef GLISSE_FWD_CASE
-        default: return cudaErrorInvalidValue;
-    }
+    diff_forward_kernel<TMAX><<<grid, kDiffBlock, 0, s>>>(a, pc, split_consts(pc));
     return cudaGetLastError();
 }
 
@@ -882,37 +973,20 @@ static int diff_task_blocks(int64_t groups, int nsm, bool force) {
 }
 
 template <int TMAX>
-static cudaError_t launch_diff_forward_tasks(int np, const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s,
+static cudaError_t launch_diff_forward_tasks(const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s,
                                              const DiffTaskArgs& b, int k, int nsm) {
-    const unsigned grid = (unsigned)(k * nsm);
     size_t smem = 0;
-    cudaError_t e = cudaSuccess;
-    switch (np) {
-#define GLISSE_FWDT_CASE(N)                                                                                  \
-    case N:                                                                                                  \
-        e = residency_cap_smem(reinterpret_cast<const void*>(diff_forward_tasks_kernel<N, TMAX>), k, 4, &smem); \
-        if (e != cudaSuccess) return e;                                                                      \
-        diff_forward_tasks_kernel<N, TMAX><<<grid, kDiffBlock, smem, s>>>(a, pc, b);                         \
-        break;
-        GLISSE_FWDT_CASE(0)
-        GLISSE_FWDT_CASE(1)
-        GLISSE_FWDT_CASE(2)
-        GLISSE_FWDT_CASE(3)
-        GLISSE_FWDT_CASE(4)
-        GLISSE_FWDT_CASE(5)
-        GLISSE_FWDT_CASE(6)
-        GLISSE_FWDT_CASE(7)
-        GLISSE_FWDT_CASE(8)
-#undef GLISSE_FWDT_CASE
-        default: return cudaErrorInvalidValue;
-    }
+    const cudaError_t e =
+        residency_cap_smem(reinterpret_cast<const void*>(diff_forward_tasks_kernel<TMAX>), k, 4, &smem);
+    if (e != cudaSuccess) return e;
+    diff_forward_tasks_kernel<TMAX><<<(unsigned)(k * nsm), kDiffBlock, smem, s>>>(a, pc, split_consts(pc), b);
     return cudaGetLastError();
 }
 
 // tb: task buffers, or null for the plain launch; force_tasks: the task launch whatever the
 // size (GLISSE_LAUNCH_TASKS).  The task launch carries no tangent or one (six keep the
 // plain launch, one block per SM).
-static cudaError_t launch_diff_forward(int np, const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s,
+static cudaError_t launch_diff_forward(const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s,
                                        const DiffTaskArgs* tb = nullptr, bool force_tasks = false) {
     if (a.n <= 0) return cudaSuccess;
     if (tb && a.ntan <= 1) {
@@ -930,18 +1004,18 @@ static cudaError_t launch_diff_forward(int np, const DiffArgs& a, const Particle
             e = cudaMemsetAsync(b.task_counter, 0, sizeof(unsigned long long), s);
             if (e == cudaSuccess) e = cudaMemsetAsync(b.group_done, 0, sizeof(int32_t) * (size_t)groups, s);
             if (e != cudaSuccess) return e;
-            return a.ntan == 0 ? launch_diff_forward_tasks<0>(np, a, pc, s, b, k, nsm)
-                               : launch_diff_forward_tasks<1>(np, a, pc, s, b, k, nsm);
+            return a.ntan == 0 ? launch_diff_forward_tasks<0>(a, pc, s, b, k, nsm)
+                               : launch_diff_forward_tasks<1>(a, pc, s, b, k, nsm);
         }
     }
-    if (a.ntan == 0) return launch_diff_forward_t<0>(np, a, pc, s);
-    if (a.ntan == 1) return launch_diff_forward_t<1>(np, a, pc, s);
-    return launch_diff_forward_t<kMaxTangents>(np, a, pc, s);
+    if (a.ntan == 0) return launch_diff_forward_t<0>(a, pc, s);
+    if (a.ntan == 1) return launch_diff_forward_t<1>(a, pc, s);
+    return launch_diff_forward_t<kMaxTangents>(a, pc, s);
 }
 
 // tb: task buffers (counter, group counters, status), or null for the plain launch.
 // force_tasks: the task launch whatever the size (GLISSE_LAUNCH_TASKS).
-static cudaError_t launch_diff_backward(int np, const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s,
+static cudaError_t launch_diff_backward(const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s,
                                         const DiffTaskArgs* tb, bool force_tasks) {
     if (a.n <= 0) return cudaSuccess;
     int dev = 0, nsm = 0;
@@ -959,46 +1033,28 @@ static cudaError_t launch_diff_backward(int np, const DiffArgs& a, const Particl
         e = cudaMemsetAsync(b.task_counter, 0, sizeof(unsigned long long), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(b.group_done, 0, sizeof(int32_t) * (size_t)groups, s);
         if (e != cudaSuccess) return e;
-        const unsigned grid = (unsigned)(k * nsm);
         size_t smem = 0;
-        switch (np) {
-#define GLISSE_DIFF_TCASE(N)                                                                                 \
-    case N:                                                                                                  \
-        e = residency_cap_smem(reinterpret_cast<const void*>(diff_backward_tasks_kernel<N>), k, 4, &smem);   \
-        if (e != cudaSuccess) return e;                                                                      \
-        diff_backward_tasks_kernel<N><<<grid, kDiffBlock, smem, s>>>(a, pc, b);                              \
-        break;
-            GLISSE_DIFF_TCASE(0)
-            GLISSE_DIFF_TCASE(1)
-            GLISSE_DIFF_TCASE(2)
-            GLISSE_DIFF_TCASE(3)
-            GLISSE_DIFF_TCASE(4)
-            GLISSE_DIFF_TCASE(5)
-            GLISSE_DIFF_TCASE(6)
-            GLISSE_DIFF_TCASE(7)
-            GLISSE_DIFF_TCASE(8)
-#undef GLISSE_DIFF_TCASE
-            default: return cudaErrorInvalidValue;
-        }
+        e = residency_cap_smem(reinterpret_cast<const void*>(diff_backward_tasks_kernel), k, 4, &smem);
+        if (e != cudaSuccess) return e;
+        diff_backward_tasks_kernel<<<(unsigned)(k * nsm), kDiffBlock, smem, s>>>(a, pc, split_consts(pc), b);
         return cudaGetLastError();
     }
     const unsigned grid = (unsigned)((a.n + kDiffBlock - 1) / kDiffBlock);
-    GLISSE_DIFF_SWITCH(diff_backward_kernel)
+    diff_backward_kernel<<<grid, kDiffBlock, 0, s>>>(a, pc, split_consts(pc));
     return cudaGetLastError();
 }
 
-static cudaError_t launch_diff_backward_growth(int np, const DiffArgs& a, const ParticleConsts& pc,
-                                               cudaStream_t s) {
+static cudaError_t launch_diff_backward_growth(const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s) {
     if (a.n <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)((a.n + kDiffBlock - 1) / kDiffBlock);
-    GLISSE_DIFF_SWITCH(diff_backward_growth_kernel)
+    diff_backward_growth_kernel<<<grid, kDiffBlock, 0, s>>>(a, pc, split_consts(pc));
     return cudaGetLastError();
 }
 
-static cudaError_t launch_diff_growth(int np, const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s) {
+static cudaError_t launch_diff_growth(const DiffArgs& a, const ParticleConsts& pc, cudaStream_t s) {
     if (a.n <= 0) return cudaSuccess;
     const dim3 grid((unsigned)((a.n + kDiffBlock - 1) / kDiffBlock), 6);
-    GLISSE_DIFF_SWITCH(diff_growth_kernel)
+    diff_growth_kernel<<<grid, kDiffBlock, 0, s>>>(a, pc, split_consts(pc));
     return cudaGetLastError();
 }
 
@@ -1037,12 +1093,12 @@ cudaError_t diff_wait_selftest(int which, int polls, char* scratch, int* status,
     if (which == 1) {
         ta.sub = kFwdSub;
         a.nsteps = 2 * kFwdSub;
-        diff_forward_tasks_kernel<0, 0><<<4, kDiffBlock, 0, s>>>(a, ParticleConsts{}, ta);
+        diff_forward_tasks_kernel<0><<<4, kDiffBlock, 0, s>>>(a, ParticleConsts{}, SplitConsts{}, ta);
     } else {
         ta.sub = kTapeSub;
         a.nsteps = 2 * kTapeSub;
         a.tape = 1;
-        diff_backward_tasks_kernel<0><<<4, kDiffBlock, 0, s>>>(a, ParticleConsts{}, ta);
+        diff_backward_tasks_kernel<<<4, kDiffBlock, 0, s>>>(a, ParticleConsts{}, SplitConsts{}, ta);
     }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1087,11 +1143,11 @@ extern "C" void glisse_diff_destroy(glisse_diff* d) { diff_free(d); }
 
 // Rows of one step's record: the drift's, the closing kick's, and with
 // GLISSE_DIFF_TAPE_TANGENT tangent 0's 9 (before the drift, and its position after).
-static int32_t rec_rows(const glisse_diff* d) { return record_rows(d->np) + (d->tan_tape ? 9 : 0); }
+static int32_t rec_rows(const glisse_diff* d) { return kScratchRows + (d->tan_tape ? 9 : 0); }
 
 static void set_record_layout(const glisse_diff* d, DiffArgs& a) {
     a.rec_rows = rec_rows(d);
-    a.tan_row = d->tan_tape ? record_rows(d->np) : 0;
+    a.tan_row = d->tan_tape ? kScratchRows : 0;
 }
 
 extern "C" int glisse_diff_checkpoint_every(glisse_diff* d, int32_t* checkpoint_every) {
@@ -1151,7 +1207,7 @@ extern "C" int glisse_diff_create(glisse_diff** out, double star_mass, const dou
             rc = GLISSE_E_CUDA;
             goto fail;
         }
-        const double tape_b = 8.0 * record_rows(n_planets) * (double)std::max<int64_t>(n_particles, 1) *
+        const double tape_b = 8.0 * kScratchRows * (double)std::max<int64_t>(n_particles, 1) *
                               (double)std::max<int64_t>(n_steps, 1);
         checkpoint_every = tape_b <= 0.5 * (double)free_b ? 0 : 256;
     }
@@ -1235,6 +1291,7 @@ extern "C" int glisse_diff_forward(glisse_diff* d, const double* state0, double*
     if (n_tangents > 0 && (!tangent0 || !tangent1)) return GLISSE_E_INVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DiffArgs a{};
+    a.np = d->np;
     a.log = d->d_log;
     a.n = d->n;
     a.nsteps = d->nsteps;
@@ -1259,7 +1316,7 @@ extern "C" int glisse_diff_forward(glisse_diff* d, const double* state0, double*
     int status = 0;
     cudaError_t e = cudaMemsetAsync(tb.status, 0, sizeof(int), s);
     if (e == cudaSuccess)
-        e = launch_diff_forward(d->np, a, d->pc, s, d->launch_mode == GLISSE_LAUNCH_PLAIN ? nullptr : &tb,
+        e = launch_diff_forward(a, d->pc, s, d->launch_mode == GLISSE_LAUNCH_PLAIN ? nullptr : &tb,
                                 d->launch_mode == GLISSE_LAUNCH_TASKS);
     if (e == cudaSuccess && removal_step && d->n > 0)
         e = cudaMemcpyAsync(removal_step, d->d_rstep, sizeof(int64_t) * d->n, cudaMemcpyDeviceToDevice, s);
@@ -1284,6 +1341,7 @@ extern "C" int glisse_diff_backward(glisse_diff* d, const double* grad_state1, d
     if (d->n > 0 && (!grad_state1 || !grad_state0)) return GLISSE_E_INVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DiffArgs a{};
+    a.np = d->np;
     a.log = d->d_log;
     a.n = d->n;
     a.nsteps = d->nsteps;
@@ -1303,7 +1361,7 @@ extern "C" int glisse_diff_backward(glisse_diff* d, const double* grad_state1, d
     int status = 0;
     cudaError_t e = cudaMemsetAsync(tb.status, 0, sizeof(int), s);
     if (e == cudaSuccess)
-        e = launch_diff_backward(d->np, a, d->pc, s, d->launch_mode == GLISSE_LAUNCH_PLAIN ? nullptr : &tb,
+        e = launch_diff_backward(a, d->pc, s, d->launch_mode == GLISSE_LAUNCH_PLAIN ? nullptr : &tb,
                                  d->launch_mode == GLISSE_LAUNCH_TASKS);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&status, tb.status, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1331,6 +1389,7 @@ extern "C" int glisse_diff_backward_growth(glisse_diff* d, const double* grad_st
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DiffArgs a{};
+    a.np = d->np;
     a.log = d->d_log;
     a.n = d->n;
     a.nsteps = d->nsteps;
@@ -1347,7 +1406,7 @@ extern "C" int glisse_diff_backward_growth(glisse_diff* d, const double* grad_st
     a.tanN = tangent1;
     a.grad0 = grad_state0;
     a.gradt0 = grad_tangent0;
-    cudaError_t e = launch_diff_backward_growth(d->np, a, d->pc, s);
+    cudaError_t e = launch_diff_backward_growth(a, d->pc, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
@@ -1363,6 +1422,7 @@ extern "C" int glisse_diff_growth_gradient(glisse_diff* d, const double* state0,
     if (d->n > 0 && (!state0 || !tangent0 || !grad_state0)) return GLISSE_E_INVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DiffArgs a{};
+    a.np = d->np;
     a.log = d->d_log;
     a.n = d->n;
     a.nsteps = d->nsteps;
@@ -1371,7 +1431,7 @@ extern "C" int glisse_diff_growth_gradient(glisse_diff* d, const double* state0,
     a.tan0 = tangent0;
     a.grad0 = grad_state0;
     a.log_growth = log_growth;
-    cudaError_t e = launch_diff_growth(d->np, a, d->pc, s);
+    cudaError_t e = launch_diff_growth(a, d->pc, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();

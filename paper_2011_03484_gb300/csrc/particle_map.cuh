@@ -109,7 +109,8 @@ __device__ __forceinline__ int kick_near(unsigned near, int np, double x, double
 // lane parity p takes planets p, p + 2, ..., the partial sums are added (the
 // same bits on both lanes: two_sum and addition commute) and the lower index wins.
 // NP: the planet count, or kAnyNp to take it from np_any (one code for all counts).
-template <int NP, int TPP>
+// WARP false: one lane by itself (*exact is the lane's own).
+template <int NP, int TPP, bool WARP = true>
 __device__ __forceinline__ int kick_sum(int np_any, double x, double y, double z, const F2 (&X)[3],
                                         const F2 (&base)[3], const Speed& sp, bool act, const double* __restrict__ L,
                                         const ParticleConsts& pc, const SplitConsts& sc, F2 (&C)[3], double (&N)[3],
@@ -140,7 +141,8 @@ __device__ __forceinline__ int kick_sum(int np_any, double x, double y, double z
     const float k2 = fmaf(C[0].h, C[0].h, fmaf(C[1].h, C[1].h, C[2].h * C[2].h));
     const bool small = k2 <= kSplitKick2 * sp.v2;
     int hit = 0;
-    exact = __any_sync(kFullMask, act && (near != 0u || !small));
+    exact = act && (near != 0u || !small);
+    if constexpr (WARP) exact = __any_sync(kFullMask, exact);
     if (exact) {
         N[0] = N[1] = N[2] = 0.0;
         if (!small) {

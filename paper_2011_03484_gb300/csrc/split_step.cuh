@@ -73,18 +73,29 @@ struct DriftFactors {
     F2 gdm1;
 };
 
-// w = 1 / r0^2 as a pair and dts = dt mu / r0^3 (mudt = mu dt) from r0^2.
-__device__ __forceinline__ void inverse_powers(double r2, double mudt, F2& w, double& dts) {
+// Scalars of drift_split for the derivatives of the drift (split_diff.cuh): those of its
+// comment, S = S + d, T = 1 - g1, rho = D - 1, rD ~ 1/D, k = (g1 - D) / D, w = 1 / r0^2 (wd: in FP64),
+// dts = dt mu / r0^3 (dts2: as a pair), fm1 = f - 1.
+struct DriftSeries {
+    F2 a, m, q, b, w, dts2, g2, g3, T, rho, D, k, fm1;
+    float rD, S, d;
+    double dts, wd;
+};
+
+// w = 1 / r0^2 as a pair (and, into wd, as a double) and dts = dt mu / r0^3 (mudt = mu dt) from r0^2.
+__device__ __forceinline__ void inverse_powers(double r2, double mudt, F2& w, double& dts, double* wd = nullptr) {
     // y ~ 1 / r0 (21 bits), e = 1 - r0^2 y^2;
     // dt mu / r0^3 = dt mu y^3 (1 - e)^(-3/2) = dt mu y^3 (1 + 3e/2 + 15e^2/8 + ...)
     const float y = __uint_as_float(__float_as_uint(rsqrt_f32(f32_trunc(r2))) & 0xFFFFFFF8u);
-    const F2 er = f2_split(fma(-r2, f21_square(y), 1.0));
+    const double y2 = f21_square(y);
+    const F2 er = f2_split(fma(-r2, y2, 1.0));
     F2 c;
     c.h = __fmul_rn(1.5f, er.h);
     c.l = __fmaf_rn(1.5f, er.l, __fmaf_rn(1.875f * er.h, er.h, __fmaf_rn(1.5f, er.h, -c.h)));
     const double dt3 = f21_kcube(y, mudt);
     dts = fma(dt3, f2_double(f2_norm(c.h, c.l)), dt3);
     // 1 / r0^2 = y^2 / (1 - e)
+    if (wd) *wd = fma(y2, f2_double(f2_norm(er.h, __fmaf_rn(er.h, er.h, er.l))), y2);
     const float yy = __fmul_rn(y, y), yl = __fmaf_rn(y, y, -yy), p = __fmul_rn(yy, er.h);
     float e;
     fast_two_sum(yy, p, w.h, e);
@@ -92,19 +103,21 @@ __device__ __forceinline__ void inverse_powers(double r2, double mudt, F2& w, do
                     __fmaf_rn(yy, __fmaf_rn(er.h, er.h, er.l), __fmaf_rn(yl, er.h, yl)));
 }
 
-// mudt = mu dt, dt2 = dt.
+// mudt = mu dt, dt2 = dt; ser (or null) receives the scalars.
 __device__ __forceinline__ bool drift_split(double r2, double mudt, double dt, const F2& dt2, const F2 (&x)[3],
-                                            const F2 (&v)[3], DriftFactors& out, Speed& sp) {
+                                            const F2 (&v)[3], DriftFactors& out, Speed& sp,
+                                            DriftSeries* ser = nullptr) {
     const F2 u = f2_dot(x, v), v2 = f2_dot(v, v);
     F2 w;
     double dts;
-    inverse_powers(r2, mudt, w, dts);
+    inverse_powers(r2, mudt, w, dts, ser ? &ser->wd : nullptr);
     float e;
     const F2 dw = f2_mul(dt2, w);
     const F2 a = f2_mul(u, dw);
     const F2 n = f2_mul(v2, f2_mul(dt2, dw));
     sp = Speed{v2.h, v2.h * w.h};
-    const F2 m = f2_mul(dt2, f2_split(dts));
+    const F2 dts2 = f2_split(dts);
+    const F2 m = f2_mul(dt2, dts2);
     const F2 q = f2_sub(n, m);
     const F2 b = f2_sub(m, q);
 
@@ -177,6 +190,10 @@ __device__ __forceinline__ bool drift_split(double r2, double mudt, double dt, c
     F2 mg2 = f2_mul(m, g2);
     mg2 = f2_norm(-mg2.h, -mg2.l);
     const F2 gd = f2_div(mg2, D, rD);
+    if (ser) {
+        const double wd = ser->wd;
+        *ser = DriftSeries{a, m, q, b, w, dts2, g2, g3, T, rho, D, k, mg2, rD, S, d, dts, wd};
+    }
     out.fm1 = f2_double(mg2);
     out.gdm1 = gd;
     out.g = fma(-dt, f2_double(f2_norm(mg3.h, mg3.l)), dt);
