@@ -88,8 +88,8 @@ extern "C" {
  * sub-chunk and then whichever group is ready, so every partition
  * keeps the same number of busy warps to the end of the segment; a warp without a
  * ready task waits (bounded: GLISSE_E_TIMEOUT after seconds).  AUTO picks TASKS when
- * the live groups outnumber the resident warps (two to five per partition) by a
- * quarter, PLAIN otherwise.  The fixed-iteration Kepler mode always uses PLAIN. */
+ * the live groups outnumber the resident warps (three to five per partition) by a
+ * tenth, PLAIN otherwise.  The fixed-iteration Kepler mode always uses PLAIN. */
 #define GLISSE_LAUNCH_AUTO 0
 #define GLISSE_LAUNCH_PLAIN 1
 #define GLISSE_LAUNCH_TASKS 2

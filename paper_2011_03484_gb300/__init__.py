@@ -719,7 +719,7 @@ class DiffMap:
     sweep alone (about half the cost); GLISSE_DIFF_AUTO takes the tape when it
     fits in half of the free device memory.  The reverse sweep for the growth
     indicator's gradient needs checkpoints, or GLISSE_DIFF_TAPE_TANGENT: a tape
-    that also keeps tangent 0 ((184 + 16 N_p) B per particle-step), after which
+    that also keeps tangent 0 (184 B per particle-step), after which
     that sweep recomputes nothing either.  The default stays K = 256."""
 
     def __init__(self, star_mass, planets, n_particles, dt, n_steps, checkpoint_every=256, **opt):

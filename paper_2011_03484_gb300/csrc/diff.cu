@@ -41,7 +41,8 @@
 // initial state needs the second derivative of the map contracted with t0.
 // diff_backward_growth_kernel gets it in one reverse sweep of the map extended
 // by its tangent (checkpoints of the state and of t), running each kick's and
-// drift's adjoint in dual numbers (state (x, t), cotangent (lt, lx));
+// drift's adjoint (state (x, t), cotangent (lt, lx)): two adjoints and the second derivative
+// in pairs (split_diff.cuh), in dual numbers for the lanes that need FP64;
 // diff_growth_kernel gets the part at fixed t0 in forward mode, one thread per
 // particle and state coordinate (used in tape mode, and as a cross-check).
 #include <cuda_runtime.h>
@@ -249,7 +250,7 @@ __device__ __forceinline__ int kick_close(int np, double (&n)[6], const F2 (&bas
 template <class T>
 __device__ __forceinline__ void kick_jac(int np, const T r[3], const double* __restrict__ L,
                                          const double (&tgm)[kMaxPlanets], const T w[3], T out[3]) {
-#pragma unroll 4
+#pragma unroll 1
     for (int j = np - 1; j >= 0; --j) {
         const T dx = r[0] - L[kRec * j], dy = r[1] - L[kRec * j + 1], dz = r[2] - L[kRec * j + 2];
         const T d2 = fma(dx, dx, fma(dy, dy, dz * dz));
@@ -261,15 +262,21 @@ __device__ __forceinline__ void kick_jac(int np, const T r[3], const double* __r
     }
 }
 
+// kick_jac_split's limit on s^2 for the orbital rate (mu / r^3)^(1/2); negative (all planets
+// near) where the position is out of the floats' range.
+__device__ __forceinline__ float near_limit(double mu, const double r[3], const F2 (&X)[3]) {
+    const int h = max(max(exp_bits(r[0]), exp_bits(r[1])), exp_bits(r[2]));
+    const float y = rsqrt_f32(fmaf(X[0].h, X[0].h, fmaf(X[1].h, X[1].h, X[2].h * X[2].h)));
+    return (unsigned)(h - (1023 - 49)) <= 98u ? kSplitNear2 * (d2f_bits(mu) * y * y * y) : -1.0f;
+}
+
 // out += tau A(r) w at the log step L, tau = dt or (half) dt / 2, w the velocity or position part of a
 // cotangent or tangent whose scale is e (ok: scale_exponent's): planets in pairs
 // (kick_jac_split), in FP64 those the particle is near to, by the rate (mu / r^3)^(1/2).
 __device__ __forceinline__ void kick_jac_add(int np, const double r[3], const F2 (&X)[3], const double* __restrict__ L,
                                              const ParticleConsts& pc, const SplitConsts& sc, bool half, bool ok,
                                              int e, const double w[3], double out[3]) {
-    const int h = max(max(exp_bits(r[0]), exp_bits(r[1])), exp_bits(r[2]));
-    const float y = rsqrt_f32(fmaf(X[0].h, X[0].h, fmaf(X[1].h, X[1].h, X[2].h * X[2].h)));
-    const float lim2 = (unsigned)(h - (1023 - 49)) <= 98u && ok ? kSplitNear2 * (d2f_bits(pc.mu) * y * y * y) : -1.0f;
+    const float lim2 = ok ? near_limit(pc.mu, r, X) : -1.0f;
     const double tau = half ? 0.5 : 1.0;
     F2 W[3], acc[3];
 #pragma unroll
@@ -278,7 +285,7 @@ __device__ __forceinline__ void kick_jac_add(int np, const double r[3], const F2
         acc[c] = F2{0.0f, 0.0f};
     }
     unsigned near = 0;
-#pragma unroll 4
+#pragma unroll 1
     for (int j = np - 1; j >= 0; --j) {
         F2 P[3];
         load_rec_split(L + kRec * j, P);
@@ -836,11 +843,115 @@ __global__ void __launch_bounds__(kDiffBlock, 4) diff_forward_tasks_kernel(const
 // then tangent 0 before the drift (6) and its position part after the drift (3).
 constexpr int kScratchRowsG = kScratchRows + 9;
 
+// The FP64 drift adjoint of the extended map for one lane, in dual numbers; rec5: as in adjoint64.
+static __device__ __noinline__ void second64(const ParticleConsts& pc, const double* pre, const double* tan,
+                                             const double* rec5, double* lt, double* lx) {
+    double x[6], t[6];
+    Dual pd[6], l[6];
+    for (int c = 0; c < 6; ++c) {
+        x[c] = pre[c];
+        t[c] = tan[c];
+        pd[c] = {x[c], t[c]};
+        l[c] = {lt[c], lx[c]};
+    }
+    DriftScalars d;
+    if (rec5[0] == 0.0) {
+        drift_scalars(pc.mu, pc.dt, x, d);
+    } else {
+        drift_restore(pc.mu, pc.dt, x, rec5[0], rec5[1], d);
+        drift_finish_stored(pc.mu, d, rec5[2], rec5[3], rec5[4]);
+    }
+    const DriftScalarsT<Dual> e = drift_lift(pc.mu, x, t, d);
+    drift_adjoint(pc.mu, pd, e, l);
+    for (int c = 0; c < 6; ++c) {
+        lt[c] = l[c].v;
+        lx[c] = l[c].d;
+    }
+}
+
+template <class T>
+__device__ __forceinline__ void swap_values(T& a, T& b) {
+    const T t = a;
+    a = b;
+    b = t;
+}
+
+// The kick of the extended map in FP64 (kick_jac in dual numbers), one lane.
+static __device__ __noinline__ void kick_second64(int np, const double* r, const double* xi, const double* L,
+                                                  const ParticleConsts& pc, bool half, double* lt, double* lx) {
+    Dual rd[3], w[3], o[3];
+    for (int c = 0; c < 3; ++c) {
+        rd[c] = {r[c], xi[c]};
+        w[c] = {lt[3 + c], lx[3 + c]};
+        o[c] = {lt[c], lx[c]};
+    }
+    kick_jac(np, rd, L, half ? pc.tgm_half : pc.tgm_full, w, o);
+    for (int c = 0; c < 3; ++c) {
+        lt[c] = o[c].v;
+        lx[c] = o[c].d;
+    }
+}
+
+// One kick's reverse step of the extended map: lt_r += tau A lt_v and
+// lx_r += tau A lx_v + tau (dA[xi]) lt_v, xi the tangent's position part; in pairs,
+// or all in FP64 for a lane that is near a planet or out of scale.
+__device__ __forceinline__ void kick_second(int np, const double r[3], const F2 (&X)[3], const double xi[3],
+                                            const double* __restrict__ L, const ParticleConsts& pc,
+                                            const SplitConsts& sc, bool half, double (&lt)[6], double (&lx)[6]) {
+    const double x6[6] = {xi[0], xi[1], xi[2], 0.0, 0.0, 0.0};
+    int et, ex, ei;
+    const bool ok = (scale_exponent(lt, et) & scale_exponent(lx, ex) & scale_exponent(x6, ei)) &&
+                    abs(et + ei) <= 900;
+    const float lim2 = near_limit(pc.mu, r, X);
+    F2 W[3], U[3], Xi[3], aW[3], aU[3], aD[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        W[c] = f2_split_scaled(lt[3 + c], ok ? et : 0);
+        U[c] = f2_split_scaled(lx[3 + c], ok ? ex : 0);
+        Xi[c] = f2_split_scaled(xi[c], ok ? ei : 0);
+        aW[c] = aU[c] = aD[c] = F2{0.0f, 0.0f};
+    }
+    bool far = ok;
+#pragma unroll 1
+    for (int j = np - 1; j >= 0; --j) {
+        F2 P[3];
+        load_rec_split(L + kRec * j, P);
+        far &= kick_second_split(X, P, sc.tg[j], lim2, W, U, Xi, aW, aU, aD);
+    }
+    if (far) {
+        const double tau = half ? 0.5 : 1.0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            lt[c] = fma(tau, f2_double_scaled(aW[c], et), lt[c]);
+            lx[c] = fma(tau, f2_double_scaled(aU[c], ex), lx[c]);
+            lx[c] = fma(tau, f2_double_scaled(aD[c], et + ei), lx[c]);
+        }
+    } else {
+        double p[3], q[3], u[6], v[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            if (c < 3) {
+                p[c] = r[c];
+                q[c] = xi[c];
+            }
+            u[c] = lt[c];
+            v[c] = lx[c];
+        }
+        kick_second64(np, p, q, L, pc, half, u, v);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            lt[c] = u[c];
+            lx[c] = v[c];
+        }
+    }
+}
+
 // One reverse sweep of the map extended by its tangent, z = (x, t) with
 // t_{k+1} = M_k(x_k) t_k, for the cotangent (lx, lt) = (grad_state1,
-// grad_growth (J t0) / |J t0|^2) at the end.  Each piece (kick, drift) runs its
-// adjoint in dual numbers: state (x, t), cotangent (lt, lx) -> (M^T lt,
-// (dM[t])^T lt + M^T lx); see drift_adjoint.  Segments are recomputed from the
+// grad_growth (J t0) / |J t0|^2) at the end.  Each piece (kick, drift) takes the
+// cotangent (lt, lx) to (M^T lt, (dM[t])^T lt + M^T lx).  ~6000 instructions a reverse step:
+// instruction fetch bounds it, so loops stay rolled (planets unrolled by four: 35 instead of
+// 21 ms; 32768 particles, 512 steps, recompute included; all in FP64: 31 ms).  Segments are recomputed from the
 // state and tangent checkpoints, as the plain backward pass does, or, with
 // GLISSE_DIFF_TAPE_TANGENT, read from the forward call's record of every step.
 // a.grad0 <- lx at t_0 (= J^T grad_state1 + grad_growth dg/dstate0 at fixed t0);
@@ -854,8 +965,11 @@ __global__ void __launch_bounds__(kDiffBlock, 2) diff_backward_growth_kernel(con
     double nn = 0.0;
     for (int c = 0; c < 6; ++c) nn = fma(a.tanN[6 * i + c], a.tanN[6 * i + c], nn);
     const double w = nn > 0.0 ? gg / nn : 0.0;
-    Dual l[6];
-    for (int c = 0; c < 6; ++c) l[c] = {w * a.tanN[6 * i + c], a.grad1 ? a.grad1[6 * i + c] : 0.0};
+    double lt[6], lx[6];
+    for (int c = 0; c < 6; ++c) {
+        lt[c] = w * a.tanN[6 * i + c];
+        lx[c] = a.grad1 ? a.grad1[6 * i + c] : 0.0;
+    }
     const int64_t rstep = a.rstep[i];
     const int reason = a.reason[i];
     const int64_t kend = rstep >= 0 ? rstep : a.nsteps;
@@ -909,30 +1023,84 @@ __global__ void __launch_bounds__(kDiffBlock, 2) diff_backward_growth_kernel(con
             }
             for (int64_t k = k1 - 1; k >= k0; --k) {
                 const double* rec = a.scratch + (k - k0) * rows * a.n + i;
-                double pre[6];
-                Dual pd[6], qd[3];
+                double pre[6], tp[6];
                 for (int c = 0; c < 6; ++c) {
                     pre[c] = rec[c * a.n];
-                    pd[c] = {pre[c], rec[(trow + c) * a.n]};
+                    tp[c] = rec[(trow + c) * a.n];
                 }
-                for (int c = 0; c < 3; ++c) qd[c] = {rec[(6 + c) * a.n], rec[(trow + 6 + c) * a.n]};
+                const double solved = rec[9 * a.n];
+                if (k > k0) {
+#pragma unroll
+                    for (int c = 0; c < 10; ++c) prefetch_l1(rec + (c - rows) * a.n);
+#pragma unroll
+                    for (int c = 0; c < 9; ++c) prefetch_l1(rec + (trow + c - rows) * a.n);
+                }
                 const bool last = (k == kend - 1);
-                if (!(last && (cut_after_drift || cut_before_drift)))
-                    kick_jac(np, qd, a.log + (k + 1) * S, (k + 1 < k1) ? pc.tgm_full : pc.tgm_half, l + 3, l);
-                if (!(last && cut_before_drift)) {
-                    DriftScalars d;
-                    const double s = rec[9 * a.n];
-                    if (s == 0.0) {
-                        drift_scalars(pc.mu, pc.dt, pre, d);
-                    } else {
-                        drift_restore(pc.mu, pc.dt, pre, s, rec[10 * a.n], d);
-                        drift_finish_stored(pc.mu, d, rec[11 * a.n], rec[12 * a.n], rec[13 * a.n]);
+                if (!(last && (cut_after_drift || cut_before_drift))) {
+                    double post[3], xi[3];
+                    for (int c = 0; c < 3; ++c) {
+                        post[c] = rec[(6 + c) * a.n];
+                        xi[c] = rec[(trow + 6 + c) * a.n];
                     }
-                    const double tp[6] = {pd[0].d, pd[1].d, pd[2].d, pd[3].d, pd[4].d, pd[5].d};
-                    const DriftScalarsT<Dual> e = drift_lift(pc.mu, pre, tp, d);
-                    drift_adjoint(pc.mu, pd, e, l);
+                    const F2 Y[3] = {f2_split(post[0]), f2_split(post[1]), f2_split(post[2])};
+                    kick_second(np, post, Y, xi, a.log + (k + 1) * S, pc, sc, k + 1 == k1, lt, lx);
                 }
-                if (k == k0) kick_jac(np, pd, a.log + k * S, pc.tgm_half, l + 3, l);
+                F2 X[3];
+                double r2;
+                split_position(pre, X, r2);
+                if (!(last && cut_before_drift)) {
+                    int et, el, ex;
+                    const bool ok = scale_exponent(tp, et) & scale_exponent(lt, el) & scale_exponent(lx, ex);
+                    if (ok && abs(et + el) <= 900 && solved == 0.0) {
+                        const F2 V[3] = {f2_split(pre[3]), f2_split(pre[4]), f2_split(pre[5])};
+                        DriftFactors f;
+                        DriftSeries ser;
+                        DriftJac J;
+                        Speed sp;
+                        drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp, &ser);
+                        drift_jac(ser, J);
+                        F2 o[6];
+                        {
+                            F2 T[2][3], L[2][3];
+#pragma unroll
+                            for (int c = 0; c < 3; ++c) {
+                                T[0][c] = f2_split_scaled(tp[c], et);
+                                T[1][c] = f2_split_scaled(tp[3 + c], et);
+                                L[0][c] = f2_split_scaled(lt[c], el);
+                                L[1][c] = f2_split_scaled(lt[3 + c], el);
+                            }
+                            drift_second_split(sc.dt, ser, J, X, V, T[0], T[1], L[0], L[1], o);
+                        }
+                        // both cotangents through one copy of the code (the loop's size is what
+                        // bounds this kernel)
+                        const int eo = et + el;
+#pragma unroll 1
+                        for (int h = 0; h < 2; ++h) {
+                            drift_adjoint_split(sc.dt, ser, f, J, pre, X, V, lx, ex);
+#pragma unroll
+                            for (int c = 0; c < 6; ++c) swap_values(lt[c], lx[c]);
+                            swap_values(el, ex);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 6; ++c) lx[c] += f2_double_scaled(o[c], eo);
+                    } else {
+                        double x[6], w[6], u[6], v[6], r5[5] = {solved, 0.0, 0.0, 0.0, 0.0};
+                        if (solved != 0.0)
+                            for (int c = 1; c < 5; ++c) r5[c] = rec[(9 + c) * a.n];
+                        for (int c = 0; c < 6; ++c) {
+                            x[c] = pre[c];
+                            w[c] = tp[c];
+                            u[c] = lt[c];
+                            v[c] = lx[c];
+                        }
+                        second64(pc, x, w, r5, u, v);
+                        for (int c = 0; c < 6; ++c) {
+                            lt[c] = u[c];
+                            lx[c] = v[c];
+                        }
+                    }
+                }
+                if (k == k0) kick_second(np, pre, X, tp, a.log + k * S, pc, sc, true, lt, lx);
             }
         }
     }
@@ -943,8 +1111,8 @@ __global__ void __launch_bounds__(kDiffBlock, 2) diff_backward_growth_kernel(con
     }
     const double w0 = n0 > 0.0 ? gg / n0 : 0.0;
     for (int c = 0; c < 6; ++c) {
-        a.grad0[6 * i + c] = l[c].d;
-        a.gradt0[6 * i + c] = fma(-w0, t0[c], l[c].v);
+        a.grad0[6 * i + c] = lx[c];
+        a.gradt0[6 * i + c] = fma(-w0, t0[c], lt[c]);
     }
 }
 

@@ -108,7 +108,10 @@ __device__ __forceinline__ int kick_near(unsigned near, int np, double x, double
 // TPP = 2: a lane pair (both lanes holding the same particle) splits the planets:
 // lane parity p takes planets p, p + 2, ..., the partial sums are added (the
 // same bits on both lanes: two_sum and addition commute) and the lower index wins.
-// NP: the planet count, or kAnyNp to take it from np_any (one code for all counts).
+// NP: the planet count, or kAnyNp to take it from np_any (one code for all counts, a rolled
+// loop: in kernels with much code the shorter loop is the faster one, 23.2 against 24.6 ms
+// for the batch's chunk unrolled by two; the unrolled one is for the single-system
+// kernels, 6.5 against 6.9 ms for 131072 particles).
 // WARP false: one lane by itself (*exact is the lane's own).
 template <int NP, int TPP, bool WARP = true>
 __device__ __forceinline__ int kick_sum(int np_any, double x, double y, double z, const F2 (&X)[3],
@@ -116,7 +119,7 @@ __device__ __forceinline__ int kick_sum(int np_any, double x, double y, double z
                                         const ParticleConsts& pc, const SplitConsts& sc, F2 (&C)[3], double (&N)[3],
                                         bool& exact) {
     const int np = NP >= 0 ? NP : np_any;
-    constexpr int kUnroll = NP >= 0 ? kMaxPlanets : 2;
+    constexpr int kUnroll = NP >= 0 ? kMaxPlanets : 1;
     const int parity = TPP == 2 ? (int)(threadIdx.x & 1) : 0;
     const float lim2 = kSplitNear2 * sp.rate2;
     load_rec_split(L + kRec * np, C);
@@ -663,14 +666,16 @@ inline cudaError_t particle_smem_cap(const void* kernel, int64_t grid, size_t* s
 //     32768 [1.7]   2.8: 2.9 | 3.1 | 3.5 | 4.8        65536 [3.4]   4.5: 4.3 | 4.0 | 4.3 | 4.5
 //     98304 [5.1]   6.9: 6.3 | 5.3 | 5.4 | 5.6       131072 [6.7]   7.5: 8.3 | 7.0 | 6.6 | 6.9
 //    262144 [13.5] 12.6: 15.7 | 12.7 | 11.8 | 11.3
-// (the last row 5 bodies).  A launch without a quarter more groups than warps is the plain one: its
-// groups would never wait for a warp, and one thread per slot needs no tickets.
+// (the last row 5 bodies).  Orbits up to e = 0.9, whose groups differ most, want more
+// warps: 57344 particles take 10.9 ms plain and 12.2 at 2 warps, 81920 12.9 and 14.1 at 3, 90112
+// 19.2 and 15.3 at 3.  So task mode starts at three warps and a tenth more groups than
+// warps (64230 live particles).
 inline int task_warps_per_partition(int64_t n, int nsteps, int n_sm) {
     const int64_t groups = (n + 31) / 32;
     const int64_t partitions = 4 * (int64_t)std::max(n_sm - 1, 1);
     if (nsteps < 2 * kSubSteps) return 0;
     const int64_t k = std::min<int64_t>(2 + groups / (3 * partitions), kTaskMaxBlocks);
-    return 4 * groups >= 5 * k * partitions ? (int)k : 0;
+    return k >= 3 && 10 * groups >= 11 * k * partitions ? (int)k : 0;
 }
 
 // tb: the task-mode buffers (counter, queue, status), or null for the plain launch.

@@ -70,6 +70,7 @@ __device__ __forceinline__ F2 f2_one_plus(const F2& x) {
 // What the tangent and the adjoint take from a drift's scalars.
 struct DriftJac {
     F2 g0, g1, iD, p, j, y, X;
+    F2 g4, g5, S;
     F2 hb0, hb1, hb2, hb3, Tb;  // -2 gb_n, -2 Tb
     F2 u;                       // dt mu / r0^5
     double tide;                // the same, FP64
@@ -88,6 +89,7 @@ __device__ __forceinline__ void drift_jac(const DriftSeries& s, DriftJac& o) {
     o.y = f2_sub(f2_sub(o.j, t1), f2_mul(s.q, f2_mul(o.p, o.p)));
     o.X = f2_add(f2_times(3.0f, s.k), f2_mul(o.p, f2_add(o.y, o.j)));
     const F2 S = f2_norm(s.S, s.d);
+    o.S = S;
     const F2 S2 = f2_mul(S, S), S4 = f2_mul(S2, S2);
     const float z = s.b.h * S2.h;
     // c4 = 1/24 - z/720 + z^2/40320, c5 = 1/120 - z/5040 + z^2/362880 (terms in z: 2^-24 of 2^-13)
@@ -97,6 +99,8 @@ __device__ __forceinline__ void drift_jac(const DriftSeries& s, DriftJac& o) {
     fast_two_sum(0.00833333377f, z * __fmaf_rn(z, 1.0f / 362880.0f, -1.0f / 5040.0f), c5.h, c5.l);
     c5.l = __fadd_rn(c5.l, -4.34617164e-10f);
     const F2 g4 = f2_mul(S4, c4), g5 = f2_mul(f2_mul(S4, S), c5);
+    o.g4 = g4;
+    o.g5 = g5;
     o.hb0 = f2_mul(S, o.g1);
     o.hb1 = f2_sub(f2_mul(S, s.g2), s.g3);
     o.hb2 = f2_sub(f2_mul(S, s.g3), F2{2.0f * g4.h, 2.0f * g4.l});
@@ -204,6 +208,91 @@ __device__ __forceinline__ void drift_adjoint_split(const F2& dt2, const DriftSe
     for (int c = 0; c < 6; ++c) l[c] = o[c];
 }
 
+// A pair and its derivative along a tangent, both pairs.
+struct D2 {
+    F2 v, d;
+};
+__device__ __forceinline__ D2 operator+(const D2& a, const D2& b) { return D2{f2_add(a.v, b.v), f2_add(a.d, b.d)}; }
+__device__ __forceinline__ D2 operator-(const D2& a, const D2& b) { return D2{f2_sub(a.v, b.v), f2_sub(a.d, b.d)}; }
+__device__ __forceinline__ D2 operator*(const D2& a, const D2& b) {
+    return D2{f2_mul(a.v, b.v), f2_add(f2_mul(a.v, b.d), f2_mul(a.d, b.v))};
+}
+__device__ __forceinline__ D2 operator*(float k, const D2& a) { return D2{f2_times(k, a.v), f2_times(k, a.d)}; }
+
+// The second derivative of the drift contracted with a tangent t = (Xi, Nu) and a cotangent
+// (Lr, Lv), all scaled pairs: o = d(M^T l)[t].  drift_adjoint_split's relations,
+// unreduced, with their derivatives: its terms are of first order in n dt and smaller, and
+// added to a sum that already holds the same products of earlier steps, so
+// that pairs serve all of them (to 2^-43 of the term against 113-bit differences).
+__device__ __forceinline__ void drift_second_split(const F2& dt2, const DriftSeries& s, const DriftJac& J,
+                                                   const F2 (&X)[3], const F2 (&V)[3], const F2 (&Xi)[3],
+                                                   const F2 (&Nu)[3], const F2 (&Lr)[3], const F2 (&Lv)[3],
+                                                   F2 (&o)[6]) {
+    const F2 dw = f2_mul(dt2, s.w);
+    const F2 al = f2_mul(s.w, f2_dot(X, Xi));
+    const F2 eta = f2_mul(dw, f2_add(f2_dot(Xi, V), f2_dot(X, Nu)));
+    const F2 kap = f2_mul(f2_mul(dt2, dw), f2_dot(V, Nu));
+    const F2 zeta = f2_add(f2_mul(s.m, al), kap);
+    const F2 sig = f2_neg(f2_mul(f2_add(f2_add(f2_mul(J.g1, al), f2_mul(s.g2, eta)), f2_mul(J.Tb, zeta)), J.iD));
+    // -2 gb4, -2 gb5 (g6 = S^6 c6, g7 = S^7 c7)
+    const float S6 = J.S.h * J.S.h * J.S.h * J.S.h * J.S.h * J.S.h;
+    const float g6 = S6 * __fmaf_rn(s.b.h, -1.0f / 40320.0f, 1.0f / 720.0f), g7 = S6 * J.S.h * (1.0f / 5040.0f);
+    const F2 hb4 = f2_sub(f2_mul(J.S, J.g5), F2{4.0f * g6, 0.0f});
+    const F2 hb5 = {__fmaf_rn(J.S.h, g6, -5.0f * g7), 0.0f};
+    const F2 e0 = f2_sub(f2_mul(J.hb0, zeta), f2_mul(f2_mul(s.b, J.g1), sig));
+    const F2 e1 = f2_add(f2_mul(J.g0, sig), f2_mul(J.hb1, zeta));
+    const F2 e2 = f2_add(f2_mul(J.g1, sig), f2_mul(J.hb2, zeta));
+    const F2 e3 = f2_add(f2_mul(s.g2, sig), f2_mul(J.hb3, zeta));
+    const F2 e4 = f2_add(f2_mul(s.g3, sig), f2_mul(hb4, zeta));
+    const F2 e5 = f2_add(f2_mul(J.g4, sig), f2_mul(hb5, zeta));
+    const F2 thD = f2_mul(J.iD, f2_add(f2_add(f2_mul(al, J.g0), e0),
+                                       f2_add(f2_mul(eta, J.g1), f2_add(f2_mul(s.a, e1), f2_mul(s.m, e2)))));
+    // the factors' derivatives
+    const F2 adt = f2_add(thD, al);
+    const F2 df = f2_mul(s.m, f2_sub(f2_mul(s.g2, al), e2));
+    const F2 dg = f2_neg(f2_mul(f2_mul(dt2, s.m), e3));
+    const F2 dfd = f2_mul(s.dts2, f2_sub(f2_mul(J.p, adt), f2_mul(J.iD, e1)));
+    const F2 dgd = f2_mul(f2_mul(s.m, J.iD), f2_sub(f2_mul(s.g2, thD), e2));
+    // total derivatives of the normalised scalars (h = dt / r0 changes too)
+    const D2 S = {J.S, f2_add(sig, f2_mul(al, J.S))};
+    const D2 g0 = {J.g0, e0}, g1 = {J.g1, f2_add(e1, f2_mul(al, J.g1))};
+    const D2 g2 = {s.g2, f2_add(e2, f2_times(2.0f, f2_mul(al, s.g2)))};
+    const D2 g3 = {s.g3, f2_add(e3, f2_times(3.0f, f2_mul(al, s.g3)))};
+    const D2 g4 = {J.g4, f2_add(e4, f2_times(4.0f, f2_mul(al, J.g4)))};
+    const D2 g5 = {J.g5, f2_add(e5, f2_times(5.0f, f2_mul(al, J.g5)))};
+    const D2 a = {s.a, f2_sub(eta, f2_times(2.0f, f2_mul(al, s.a)))};
+    const D2 m = {s.m, f2_times(-3.0f, f2_mul(al, s.m))};
+    const D2 b = {s.b, f2_times(2.0f, f2_sub(f2_mul(al, f2_sub(s.q, f2_times(2.0f, s.m))), kap))};
+    const D2 iD = {J.iD, f2_mul(J.iD, f2_sub(al, thD))};
+    // the adjoint
+    const F2 dtt = f2_mul(dt2, dt2);
+    const D2 lf = {f2_mul(dt2, f2_dot(Lr, X)), f2_mul(dt2, f2_dot(Lr, Xi))};
+    const D2 lg = {f2_mul(dtt, f2_dot(Lr, V)), f2_mul(dtt, f2_dot(Lr, Nu))};
+    const D2 PiD = iD * D2{f2_dot(Lv, X), f2_dot(Lv, Xi)};
+    const D2 tL = iD * D2{f2_mul(dt2, f2_dot(Lv, V)), f2_mul(dt2, f2_dot(Lv, Nu))};
+    const D2 c0 = iD * (PiD * g1 + tL * g2);
+    const D2 c1 = c0 * a - PiD;
+    const D2 c2 = c0 * m - (lf + tL);
+    const D2 e = iD * (g0 * c1 + g1 * (c2 - b * c0) - g2 * lg);
+    const D2 hb1 = S * g2 - g3, hb2 = S * g3 - 2.0f * g4, hb3 = S * g4 - 3.0f * g5;
+    const D2 H = S * g1 * c0 + hb1 * c1 + hb2 * c2 - hb3 * lg - (hb1 + a * hb2 + m * hb3) * e;
+    const D2 ca = g2 * lf + g1 * (PiD - e) + g0 * c0 + m * H;
+    const D2 ce = g1 * c0 - g2 * e;
+    const D2 u = {J.u, f2_times(-5.0f, f2_mul(al, J.u))};
+    const D2 ua = u * ca;
+    const D2 ud = {f2_mul(dt2, u.v), f2_mul(dt2, u.d)}, ue = ud * ce;
+    const D2 uk = D2{f2_mul(dt2, ud.v), f2_mul(dt2, ud.d)} * H;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        o[c] = f2_add(f2_add(f2_add(f2_mul(df, Lr[c]), f2_mul(dfd, Lv[c])),
+                             f2_add(f2_mul(ua.d, X[c]), f2_mul(ua.v, Xi[c]))),
+                      f2_add(f2_mul(ue.d, V[c]), f2_mul(ue.v, Nu[c])));
+        o[3 + c] = f2_add(f2_add(f2_add(f2_mul(dg, Lr[c]), f2_mul(dgd, Lv[c])),
+                                 f2_add(f2_mul(ue.d, X[c]), f2_mul(ue.v, Xi[c]))),
+                          f2_add(f2_mul(uk.d, V[c]), f2_mul(uk.v, Nu[c])));
+    }
+}
+
 // One planet's share of the tidal matrix of a full kick, dt A w = -s (w - 3 d (d.w) / |d|^2) with
 // s = dt G m / |d|^3, added to acc (w: the scaled pairs W).  False, adding nothing, when
 // the planet is near (as in kick_split): the caller then forms the term in FP64.
@@ -221,6 +310,35 @@ __device__ __forceinline__ bool kick_jac_split(const F2 (&x)[3], const F2 (&P)[3
     const F2 t = f2_mul(f2_mul(s, inv), f2_times(3.0f, f2_dot(d, W)));
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[c] = f2_add(acc[c], f2_sub(f2_mul(t, d[c]), f2_mul(s, W[c])));
+    return far;
+}
+
+// The same for two cotangents W, U and the matrix's derivative along Xi applied to W,
+//   d(dt A)[xi] w = 3 s (mu w + la xi + (xi.w / |d|^2 - 5 mu la) d),  mu = d.xi / |d|^2, la = d.w / |d|^2:
+// accW, accU += dt A w, dt A u; accD += d(dt A)[xi] w.
+__device__ __forceinline__ bool kick_second_split(const F2 (&x)[3], const F2 (&P)[3], const F2& tg, float lim2,
+                                                  const F2 (&W)[3], const F2 (&U)[3], const F2 (&Xi)[3],
+                                                  F2 (&accW)[3], F2 (&accU)[3], F2 (&accD)[3]) {
+    F2 d[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d[c] = f2_sub(x[c], P[c]);
+    const RsqrtF2 r = f2_rsqrt(f2_norm2(d));
+    F2 s = f2_k_rcube(r, tg);
+    const bool far = s.h * s.h <= lim2;
+    s.h = far ? s.h : 0.0f;
+    s.l = far ? s.l : 0.0f;
+    const F2 inv = {far ? r.yy : 0.0f, far ? __fmaf_rn(r.yy, r.e * __fadd_rn(1.0f, r.e), r.yl) : 0.0f};
+    const F2 s3 = f2_times(3.0f, s);
+    const F2 la = f2_mul(inv, f2_dot(d, W)), mu = f2_mul(inv, f2_dot(d, Xi));
+    const F2 tw = f2_mul(s3, la), tu = f2_mul(s3, f2_mul(inv, f2_dot(d, U)));
+    const F2 tm = f2_mul(s3, mu);
+    const F2 td = f2_mul(s3, f2_sub(f2_mul(inv, f2_dot(Xi, W)), f2_times(5.0f, f2_mul(mu, la))));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        accW[c] = f2_add(accW[c], f2_sub(f2_mul(tw, d[c]), f2_mul(s, W[c])));
+        accU[c] = f2_add(accU[c], f2_sub(f2_mul(tu, d[c]), f2_mul(s, U[c])));
+        accD[c] = f2_add(accD[c], f2_add(f2_add(f2_mul(tm, W[c]), f2_mul(tw, Xi[c])), f2_mul(td, d[c])));
+    }
     return far;
 }
 

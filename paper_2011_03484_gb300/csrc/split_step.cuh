@@ -111,7 +111,6 @@ __device__ __forceinline__ bool drift_split(double r2, double mudt, double dt, c
     F2 w;
     double dts;
     inverse_powers(r2, mudt, w, dts, ser ? &ser->wd : nullptr);
-    float e;
     const F2 dw = f2_mul(dt2, w);
     const F2 a = f2_mul(u, dw);
     const F2 n = f2_mul(v2, f2_mul(dt2, dw));

@@ -346,7 +346,7 @@ def test_split_invariance(G, orc):
 
 @pytest.mark.parametrize("name,n,steps,opt", [
     ("longrun", 131072, 2100, {}),                                   # AUTO picks tasks; first-chunk pieces
-    ("longrun", 49152, 97, {}),                                      # two warps per partition, ragged sub-chunk
+    ("longrun", 65536, 97, {}),                                      # the smallest AUTO launches as tasks, ragged
     ("longrun", 33, 300, {}),
     ("longrun", 1025, 700, {"chunk_steps": 128, "resync_chunks": 3}),
     ("eccentric", 4096, 900, {"chunk_steps": 256}),                  # removals, general-solver lanes
