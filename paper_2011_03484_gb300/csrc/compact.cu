@@ -6,8 +6,8 @@
 // copied, in order, into a second set of planes:
 //   1. count: live entries per tile of kTile slots
 //   2. scan:  exclusive prefix of the tile counts (one block), total -> n_out
-//   3. scatter: per tile, rounds of 256 slots; a warp ballot ranks the live
-//      slots inside a warp, warp totals rank warps inside the block, and the
+//   3. scatter: per tile, a warp takes 256 consecutive slots; ballots rank the live
+//      slots inside the warp, warp totals rank warps inside the block, and the
 //      tile offset places the block; each live slot writes its six state
 //      values and its id.
 // The pass is bound by HBM traffic: 8 x 6 + 4 bytes read and written per
@@ -100,31 +100,49 @@ __global__ void __launch_bounds__(kCompactThreads) compact_scatter_kernel(
     const double* __restrict__ src,
     const int32_t* __restrict__ src_id, int64_t lds, double* __restrict__ dst, int32_t* __restrict__ dst_id,
     int64_t ldd) {
+    // a warp holds kCompactRounds consecutive runs of 32 slots: their ballots place every slot
+    // after one exchange between the warps, and the copies then run without a barrier,
+    // kBatch runs' loads in flight
+    constexpr int kBatch = 4;
     __shared__ int wcnt[kCompactThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int64_t out = offsets[blockIdx.x];
-    const int64_t base = (int64_t)blockIdx.x * kTile;
+    const int64_t base = (int64_t)blockIdx.x * kTile + warp * (32 * kCompactRounds) + lane;
+    unsigned ball[kCompactRounds];
+    int cnt = 0;
+#pragma unroll
     for (int r = 0; r < kCompactRounds; ++r) {
-        const int64_t idx = base + r * kCompactThreads + threadIdx.x;
-        const bool f = idx < n && selected(key[idx], want);
-        const unsigned ball = __ballot_sync(0xFFFFFFFFu, f);
-        const int rank = __popc(ball & ((1u << lane) - 1u));
-        if (lane == 0) wcnt[warp] = __popc(ball);
-        __syncthreads();
-        int woff = 0, tot = 0;
+        const int64_t idx = base + 32 * r;
+        ball[r] = __ballot_sync(0xFFFFFFFFu, idx < n && selected(key[idx], want));
+        cnt += __popc(ball[r]);
+    }
+    if (lane == 0) wcnt[warp] = cnt;
+    __syncthreads();
+    int64_t out = offsets[blockIdx.x];
 #pragma unroll
-        for (int w = 0; w < kCompactThreads / 32; ++w) {
-            woff += (w < warp) ? wcnt[w] : 0;
-            tot += wcnt[w];
-        }
-        if (f) {
-            const int64_t d = out + woff + rank;
+    for (int w = 0; w < kCompactThreads / 32; ++w) out += (w < warp) ? wcnt[w] : 0;
 #pragma unroll
-            for (int c = 0; c < 6; ++c) dst[c * ldd + d] = src[c * lds + idx];
-            dst_id[d] = src_id[idx];
+    for (int r0 = 0; r0 < kCompactRounds; r0 += kBatch) {
+        double v[kBatch][6];
+        int32_t id[kBatch];
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+            const int64_t idx = base + 32 * (r0 + q);
+            if ((ball[r0 + q] >> lane) & 1u) {
+#pragma unroll
+                for (int c = 0; c < 6; ++c) v[q][c] = src[c * lds + idx];
+                id[q] = src_id[idx];
+            }
         }
-        out += tot;
-        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+            if ((ball[r0 + q] >> lane) & 1u) {
+                const int64_t d = out + __popc(ball[r0 + q] & ((1u << lane) - 1u));
+#pragma unroll
+                for (int c = 0; c < 6; ++c) dst[c * ldd + d] = v[q][c];
+                dst_id[d] = id[q];
+            }
+            out += __popc(ball[r0 + q]);
+        }
     }
 }
 
