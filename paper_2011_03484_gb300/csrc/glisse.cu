@@ -71,18 +71,20 @@ constexpr size_t kRingBudgetBytes = size_t(512) << 20;
 constexpr int64_t kEphQueue = 8;
 // The first chunk of planets has no particle work to overlap with.  Its kernel
 // publishes its step count to host-mapped memory, and the particles of that chunk
-// run in segments ending at steps kFirstPiece * g^k, each launched once the host
-// sees its planet steps written: the particles follow the planets from the first
-// piece on, while the planet kernel keeps its SM.  A piece g times as long as the
-// steps before it never waits for its planets when a particle step takes at least
-// g planet steps: g = 4 when the particles fill kFourfoldWarps warps per SM
-// partition or more (a planet step is ~1.2 warp-steps of particles on a partition:
-// ~146 against ~109 FP64 instructions, at a busier pipe), else g = 2.  Fewer
-// pieces mean fewer launch tails (measured on 131072 particles: the first chunk
-// 26.41 ms with g = 4 against 26.75 ms with g = 2).
-constexpr int kMaxPieces = 8;
+// run in segments, each launched once the host sees its planet steps written: the
+// particles follow the planets from step kFirstPiece on, while the planet kernel
+// keeps its SM.  A piece that ends at g times the step it starts at never waits for
+// its planets when a particle step takes at least g planet steps, and fewer pieces
+// mean fewer launch tails.  A planet step takes 2.4 us, a particle step 2.0 us with one
+// warp per SM partition, 3.9 with three, 5.3 with five, 9.5 with ten: from kFourfoldWarps on
+// g = 4, from kTwofoldWarps on g = 2, below that pieces of kPieceSteps steps (doubling up to
+// there), since the last one then runs after the last planet step.  The call that advances
+// a new context by 1024 steps (ms, before: g = 4 from five warps on, else 2): 1024
+// particles 3.4 -> 2.9, 32768 3.7 -> 3.1, 49152 4.4 -> 4.1, 98304 6.3 -> 5.5.
+constexpr int kMaxPieces = 48;  // the most that any chunk length gives is 40
 constexpr int64_t kFirstPiece = kProgressEvery;
-constexpr int64_t kFourfoldWarps = 5;
+constexpr int64_t kPieceSteps = 128;
+constexpr int64_t kTwofoldWarps = 3, kFourfoldWarps = 10;
 // A count that has not arrived after this long means the GPU is busy with other
 // work (the planet kernel has not started): the rest of the chunk then waits for
 // the planet kernel's completion event instead.  The longest piece the host polls
@@ -306,12 +308,13 @@ static int ensure_chunk(glisse_ctx* c, int64_t j) {
             GL_CUDA(cudaGetDevice(&dev));
             GL_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
             const int64_t partitions = 4 * (int64_t)std::max(nsm - 1, 1);  // the ephemeris holds one SM
-            const int shift = c->n_live >= kFourfoldWarps * 32 * partitions ? 2 : 1;
+            const int64_t warps = c->n_live / (32 * partitions);
+            // longest piece: none for g = 2, 4; else kPieceSteps, or a sixteenth of a long chunk
+            const int64_t most = warps >= kTwofoldWarps ? c->C : std::max<int64_t>(kPieceSteps, c->C / 16);
+            const int64_t g = warps >= kFourfoldWarps ? 4 : 2;
             c->n_pieces = 0;
-            for (int64_t b = 0; b < c->C; b = c->piece_end[c->n_pieces++])
-                c->piece_end[c->n_pieces] = c->n_pieces == kMaxPieces - 1
-                                                ? c->C
-                                                : std::min<int64_t>(c->C, kFirstPiece << (shift * c->n_pieces));
+            for (int64_t b = 0, e = kFirstPiece; b < c->C; b = e, e = std::min<int64_t>(g * b, b + most))
+                c->piece_end[c->n_pieces++] = std::min<int64_t>(c->C, e);
             prog = c->d_prog;
         }
         if (c->np > 0)
@@ -335,10 +338,12 @@ static int ensure_chunk(glisse_ctx* c, int64_t j) {
 // glisse_advance call can enqueue the planets of all its chunks at once: the
 // planet kernel then runs ahead while the particles are the slower stage and
 // has the log ready when they become the faster one (few live particles).
-// Between calls nothing of the main stream is in flight; the side stream is
-// drained, and slots holding chunks move (pointers and events) to the position
-// of their chunk in the larger ring.  An allocation failure keeps the ring as
-// it is (the lookahead is an optimisation).
+// Between calls nothing of the main stream is in flight.  Slots holding chunks move
+// (pointers and events; a planet kernel in flight writes to the same buffers, and is not
+// waited for: that wait was 2.4 ms at the start of a new context's first long call) to the
+// position of their chunk in the larger ring: chunks in the ring are consecutive, so
+// that no two of them meet.  An allocation failure keeps the ring as it is (the lookahead
+// is an optimisation).
 static int grow_ring(glisse_ctx* c, size_t want) {
     const size_t cap = std::max(kRingMin, kRingBudgetBytes / std::max<size_t>(slot_bytes(c), 1));
     want = std::min(want, cap);
@@ -351,7 +356,6 @@ static int grow_ring(glisse_ctx* c, size_t want) {
             return GLISSE_OK;
         }
     }
-    GL_CUDA(cudaStreamSynchronize(c->se));
     std::vector<Slot> next(want);
     std::vector<Slot> spare;
     for (Slot& old : c->ring) {
@@ -812,7 +816,7 @@ extern "C" int glisse_advance(glisse_ctx* c, int64_t n_steps) {
         return rc;
     // the planets may run ahead of the particles up to the call's last chunk (+1)
     const int64_t j_last = c->external ? 0 : (c->step + n_steps - 1) / c->C;
-    if (!c->external && (rc = grow_ring(c, (size_t)(j_last - c->step / c->C + kRingMin))) != GLISSE_OK) return rc;
+    if (!c->external && (rc = grow_ring(c, (size_t)(j_last - c->step / c->C + 2))) != GLISSE_OK) return rc;
     while (remaining > 0 && rc == GLISSE_OK) {
         const double* log = nullptr;
         int64_t m = 0;

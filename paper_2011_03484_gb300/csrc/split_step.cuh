@@ -7,11 +7,10 @@
 // One step then takes 19 FP64 instructions (r^2 and dt mu / r^3: 5; g, fdot: 2;
 // f x + g v: 6; fdot x: 3; gdot v and the kick, summed in pairs: 3) against 61 + 12 N_p for
 // the all-FP64 step, and ~1200 instructions in all, which fit under them.
-// Measured (1048576 particles, 4 planets, 1024 steps): 53 ms against 207 ms, FP64
-// pipe 81% busy, issue slots 58%.  Against 113-bit arithmetic, one step's velocity is
-// off by 0.73 to 0.95 units of 2^-53 (rms over belts of 20-100 AU; the all-FP64 step:
-// 1.09 to 1.21) and its energy by 1.6 to 1.75 (2.1 to 2.4): fewer roundings, and
-// what the pairs drop lies below them.
+// Measured (1048576 particles, 4 planets, 1024 steps): 44.8 ms against 207 ms; the 19
+// instructions at 65 cycles are 73% of that.  Against 113-bit arithmetic, one step's velocity
+// is off by 0.58 to 0.71 units of 2^-53 (rms over belts of 20-100 AU; the all-FP64 step:
+// 1.09 to 1.21): fewer roundings, and what the pairs drop lies below them.
 #pragma once
 #include "glisse_internal.h"
 #include "split_math.cuh"
@@ -48,7 +47,7 @@ __host__ __device__ inline void split_step_consts(const ParticleConsts& pc, Spli
 // so the factors of x and v come from pairs except for dt and dt mu / r0^3, which
 // are FP64.  S: series start, one Newton step in FP32, one in pairs (the error
 // left is below (a/2) (2^-18)^2).
-// Domain: |a| <= 2^-5, b and m <= kSplitZ; the caller runs the FP64 drift for
+// Domain: |a| <= kSplitA, b and m <= kSplitZ; the caller runs the FP64 drift for
 // other lanes.
 // ---------------------------------------------------------------------------
 constexpr float kSplitZ = 0.00390625f;  // 2^-8
