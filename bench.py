@@ -36,17 +36,16 @@ METRIC = "FP64 particle-steps/s at 1 GB300 (4 planets, 1e5-1e6 particles); % FP6
 UNIT = "particle-steps/s"
 
 # FP64 work of one interior particle-step in the kernel's formulation (static count of
-# the source; ncu's executed DADD:DMUL:DFMA mix matches it): the fast Kepler drift with
-# the degree-3 Stumpff tier (3 DADD, 13 DMUL, 42 DFMA), the h0 term (3 DFMA), and per
-# planet 3 DADD + 1 DMUL + 8 DFMA (separation, |d|^2, k |d|^-3 with the seed's square
-# and k times its cube formed in integer arithmetic, velocity update).
+# the source): |r|^2 3, dt mu / |r|^3 2, g and fdot 2, x' = f x + g v 6, v + fdot x 3, and
+# one sum of the velocity with the drift's and the kick's corrections, which are float pairs, 3.
 def fp64_instr_per_step(np_: int) -> int:
-    return 58 + 3 + 12 * np_
+    # the same for every planet count: the kick enters as float pairs, in one sum per component
+    return 19
 
 
 def flop_per_step(np_: int) -> int:
-    # DFMA counts 2 FLOP, DADD / DMUL 1
-    return (3 + 13 + 2 * 42) + 2 * 3 + np_ * (3 + 1 + 2 * 8)
+    # DFMA counts 2 FLOP, DADD / DMUL 1: 3 DADD + 1 DMUL + 15 DFMA
+    return 3 + 1 + 2 * 15
 
 
 # GB300 FP64 pipe: 2 DFMA per clock per SM (ncu: sm__sass_thread_inst_executed_op_dfma_pred_on
@@ -55,7 +54,8 @@ DFMA_PER_CLK_PER_SM = 2
 
 
 PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "particle_tasks_kernel_longrun.txt")
-KERNEL_SOURCES = ["particle_map.cuh", "particles.cu", "kepler.cuh", "device_math.cuh", "glisse_internal.h"]
+KERNEL_SOURCES = ["particle_map.cuh", "particles.cu", "split_step.cuh", "split_math.cuh", "kepler.cuh", "device_math.cuh",
+                  "glisse_internal.h"]
 
 
 def kernel_hash() -> str:
@@ -856,7 +856,7 @@ def main():
                    "parallelism": f"replicas x{world} (independent particle sets, no collective)",
                    "wall_s": r["t_wall"]},
         "kepler": (f"paper fixed-iteration solve, {args.kepler_iters} Newton iterations (library sin/cos)"
-                   if paper else "converged (FP32 pre-solve + FP64 Halley step)"),
+                   if paper else "converged (float-pair corrections to FP64 sums; FP64 solve outside their domain)"),
         "sampling": (f"barycentric elements + 3:2 libration test every {args.sample_every} steps"
                      if args.sample_every > 0 else None),
         "sort": "by expected Kepler-solve cost, costliest first" if args.sort else None,
@@ -865,8 +865,9 @@ def main():
             "frac": achieved / peak, "traffic": traffic,
             "kernel": "particle_tasks_kernel<4> (the task launch AUTO picks for this workload)",
             "kernel_ms_avg": kernel_ms, "flop_per_particle_step": flop_per_step(np_),
-            "flop_count": "the kernel's own FP64 work per particle-step (static count, equal to ncu's "
-                          "executed DADD/DMUL/DFMA mix); the oracle's count is given beside it",
+            "flop_count": "the kernel's own FP64 work per particle-step (static count of the usual path; its "
+                          "~1200 FP32 and integer instructions are not counted); the oracle's count is given "
+                          "beside it",
             "flop_per_particle_step_oracle": orc_flop,
             "frac_at_oracle_count": (orc_flop * steps_per_launch / (kernel_ms * 1e-3) / peak) if orc_flop else None,
             "fp64_instr_per_particle_step": fp64_instr_per_step(np_), "fp64_pipe_frac": pipe,

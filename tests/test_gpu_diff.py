@@ -128,6 +128,32 @@ def test_adjoint_is_the_transpose_of_the_tangent(G):
     assert rel.max() < 1e-11
 
 
+@pytest.mark.parametrize("every", [0, 16])
+def test_cotangent_scale(G, every):
+    """Cotangents enter the float pairs divided by the power of two of their largest component:
+    J^T (2^k g) is 2^k J^T g bit for bit up to 2^800, beyond 2^900 (FP64 instead) to rounding,
+    and a zero cotangent gives zeros.  Planet-crossing orbits up to e = 0.9, so that pairs
+    and the lanes solved in FP64 both take part."""
+    n, steps = 257, 40
+    _, pl, _ = _workload(8)
+    s0 = _cuda(gi.particle_belt(np.random.default_rng(5), n, (20.0, 30.0), (0.0, 0.9), 2.0))
+    dm = G.DiffMap(1.0, pl, n, 0.5, steps, checkpoint_every=every)
+    dm.forward(s0)
+    g = np.random.default_rng(6).standard_normal((n, 6))
+    base = dm.backward(_cuda(g)).cpu().numpy()
+    for k in (-800, 1, 800):
+        np.testing.assert_array_equal(dm.backward(_cuda(np.ldexp(g, k))).cpu().numpy(), np.ldexp(base, k))
+    norm = np.abs(base).max(axis=1, keepdims=True)
+    for k in (-950, 950):
+        got = np.ldexp(dm.backward(_cuda(np.ldexp(g, k))).cpu().numpy(), -k)
+        # two formulations, each good to some 2^-50 of the vector a step; what a step leaves grows,
+        # against the vector itself, by at most the condition of the map between apocentre and
+        # pericentre, about their ratio (19 at e = 0.9) cubed
+        assert (np.abs(got - base) <= steps * 2.0**-50 * 19.0**3 * norm).all(), (np.abs(got - base) / norm).max()
+    assert (dm.backward(_cuda(np.zeros((n, 6)))).cpu().numpy() == 0.0).all()
+    dm.close()
+
+
 def test_gradient_independent_of_checkpoint_interval(G):
     """Interior kicks merge inside a checkpoint segment and stay half kicks at its
     boundaries, so the trajectory, and with it the gradient, depends on K only by

@@ -81,6 +81,33 @@ def test_planet_ephemeris_parity(G, orc, n_steps):
     np.testing.assert_array_equal(g["planets"][:, 0], w["planets"][:, 0])
 
 
+@pytest.mark.parametrize("mass,sep", [(3e-3, 0.15), (1e-5, 0.02), (1e-2, 0.6)])
+def test_heavy_or_close_planets(G, orc, mass, sep):
+    """Planets whose mutual kick is too strong for float pairs (summed in FP64 instead), or
+    nearly: two of them, `sep` apart in semi-major axis, over 300 steps against the oracle,
+    within what rounding-sized changes of the planets' input do to the oracle's own run."""
+    dt, n = 0.02, 300
+    G_ = gi.G
+    pl = np.zeros((2, 7))
+    for j, (a, ph) in enumerate(((1.0, 0.0), (1.0 + sep, 0.6))):
+        st = gi.elements_to_cartesian(G_ * (1 + mass), np.array([a]), np.array([0.02]), np.array([0.01]),
+                                      np.array([0.1]), np.array([0.2]), np.array([ph]))[0]
+        pl[j] = np.concatenate([[mass], st])
+    w = {"star_mass": 1.0, "planets": pl, "particles": gi.make("tiny", n=2)["particles"], "dt": dt}
+    got = run_gpu(G, w, n)["planets"][:, 1:]
+    ref = orc.planet_wh(1.0, pl, dt, n, want_log=False)[0][:, 1:]
+    sens = 0.0
+    rng = np.random.default_rng(3)
+    for _ in range(8):
+        q = pl.copy()
+        q[:, 1:] *= 1 + 2.0**-52 * rng.integers(-1, 2, (2, 6))
+        sens = max(sens, parity.rel_err(orc.planet_wh(1.0, q, dt, n, want_log=False)[0][:, 1:], ref).max())
+    e = parity.rel_err(got, ref).max()
+    bound = parity.sens_factor(n) * max(sens, 2.0**-52)
+    print(f"mass {mass} sep {sep}: {e:.2e} (bound {bound:.2e})")
+    assert e <= bound, (e, bound)
+
+
 def test_planet_log_chunking_is_exact(G):
     """The planet sequence does not depend on the chunk length (bitwise)."""
     w = gi.make("tiny", n=4)
@@ -103,8 +130,8 @@ def test_first_chunk_pieces_are_exact(G):
 
 def test_first_chunk_piece_schedules_agree(G):
     """The 131072-particle context fills more than five warps per SM partition, so its first
-    chunk runs in pieces growing four-fold (16, 64, 256, 1024 steps), mostly as task launches;
-    a context holding only its first 32768 particles runs pieces growing two-fold, as plain
+    chunk runs in pieces growing two-fold (16, 32, ..., 1024 steps), mostly as task launches;
+    a context holding only its first 32768 particles runs pieces of at most 128 steps, as plain
     launches.  Particles are independent and every cut is open, so the shared particles end
     the first chunk bit-identical (before any compaction changes who shares a warp)."""
     w = gi.make("longrun")
