@@ -457,11 +457,12 @@ __global__ void __launch_bounds__(kDiffBlock) diff_growth_kernel(const DiffArgs 
     const int c = blockIdx.y;
     if (i >= a.n) return;
     const int np = a.np, S = log_stride(np);
-    double st[6], dx[6], tv[1][6];  // tv: the forward pass's tangent, bit for bit, as t's value
+    // tv[0]: the forward pass's tangent, bit for bit, as t's value; tv[1]: dx
+    double st[6], tv[2][6];
     Dual t[6];
     for (int k = 0; k < 6; ++k) {
         st[k] = a.state0[6 * i + k];
-        dx[k] = (k == c) ? 1.0 : 0.0;
+        tv[1][k] = (k == c) ? 1.0 : 0.0;
         t[k] = {a.tan0[6 * i + k], 0.0};
         tv[0][k] = t[k].v;
     }
@@ -479,24 +480,23 @@ __global__ void __launch_bounds__(kDiffBlock) diff_growth_kernel(const DiffArgs 
         const double* L0 = a.log + k * S;
         const double* L1 = L0 + S;
         if (!opened) {
-            const Dual rd[3] = {{st[0], dx[0]}, {st[1], dx[1]}, {st[2], dx[2]}};
+            const Dual rd[3] = {{st[0], tv[1][0]}, {st[1], tv[1][1]}, {st[2], tv[1][2]}};
             kick_jac(np, rd, L0, pc.tgm_half, t, t + 3);
-            kick_jac(np, st, L0, pc.tgm_half, dx, dx + 3);
-            kick_jac_tangent(np, st, X, L0, pc, sc, true, tv[0]);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) kick_jac_tangent(np, st, X, L0, pc, sc, true, tv[q]);
             kick_open(np, st, X, r2, L0, pc, sc);
         }
         double pdx[6], n[6];
         for (int q = 0; q < 6; ++q) {
-            pdx[q] = dx[q];
+            pdx[q] = tv[1][q];
             t[q].v = tv[0][q];
         }
         F2 base[3];
         Speed sp;
         DriftScalars d;
-        if (diff_drift<1, 1>(pc, sc, st, X, r2, n, base, sp, tv, nullptr, 0) ||
+        if (diff_drift<2, 2>(pc, sc, st, X, r2, n, base, sp, tv, nullptr, 0) ||
             !drift_scalars(pc.mu, pc.dt, st, d))
             break;
-        drift_tangent(pc.mu, st, d, dx);
         {
             const DriftScalarsT<Dual> e = drift_lift(pc.mu, st, pdx, d);
             Dual pd[6];
@@ -511,10 +511,10 @@ __global__ void __launch_bounds__(kDiffBlock) diff_growth_kernel(const DiffArgs 
         const double(&tgm)[kMaxPlanets] = merge ? pc.tgm_full : pc.tgm_half;
         split_position(st, X, r2);
         if (kick_close(np, st, base, sp, X, r2, merge, L1, pc, sc)) break;
-        const Dual rd[3] = {{st[0], dx[0]}, {st[1], dx[1]}, {st[2], dx[2]}};
+        const Dual rd[3] = {{st[0], tv[1][0]}, {st[1], tv[1][1]}, {st[2], tv[1][2]}};
         kick_jac(np, rd, L1, tgm, t, t + 3);
-        kick_jac(np, st, L1, tgm, dx, dx + 3);
-        kick_jac_tangent(np, st, X, L1, pc, sc, !merge, tv[0]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) kick_jac_tangent(np, st, X, L1, pc, sc, !merge, tv[q]);
         opened = merge;
     }
     double n1 = 0.0, p1 = 0.0;
