@@ -1057,7 +1057,7 @@ __global__ void __launch_bounds__(kDiffBlock, 2) diff_backward_growth_kernel(con
                         DriftSeries ser;
                         DriftJac J;
                         Speed sp;
-                        drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp, &ser);
+                drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp, &ser);
                         drift_jac(ser, J);
                         F2 o[6];
                         {

@@ -167,13 +167,6 @@ __device__ __forceinline__ int kick_sum(int np_any, double x, double y, double z
 
 __device__ __forceinline__ double f2_sum(const F2& v) { return f2_double(f2_norm(v.h, v.l)); }
 
-// drift_wide out of line (few warps need it: its registers and code stay off the usual path).
-static __device__ __noinline__ bool drift_wide_call(double r2, double mudt, double dt, F2 dt2, double x, double y,
-                                                    double z, double vx, double vy, double vz, DriftFactors& f) {
-    const double s[6] = {x, y, z, vx, vy, vz};
-    return drift_wide(r2, mudt, dt, dt2, s, f);
-}
-
 // The FP64 drift (kepler.cuh) of the lanes that the pairs leave (part): the fast
 // path, then the general solver for lanes outside its domain.  Returns false for a
 // lane whose solve failed.  All lanes of a warp call it together.
@@ -262,6 +255,7 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
         }
     }
 
+    bool all_slow = false;
     for (int k = 0; k < nsteps; ++k) {
         if (!__any_sync(kFullMask, act)) break;
         const double* __restrict__ Ln = L + (size_t)(k + 1) * S;
@@ -273,22 +267,16 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
         Speed sp;
         if constexpr (MODE == kDriftConverge) {
             const F2 V[3] = {f2_split(vx), f2_split(vy), f2_split(vz)};
-            DriftFactors f;
-            bool slow = !drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp) && act;
+            DriftFactors f = {0.0, 0.0, 0.0, kZero};
+            bool slow = act;
+            // a warp whose lanes all stepped too far for the pairs spares itself the attempt while
+            // m alone says so (same results: those lanes take the FP64 drift either way)
+            if (!all_slow || __any_sync(kFullMask, act && !beyond_split(r2, d2f_bits(sc.mudt), sc.dt.h)))
+                slow = !drift_split(r2, sc.mudt, pc.dt, sc.dt, X, V, f, sp) && act;
+            else
+                sp = split_speed(r2, sc.mudt, V);
 #pragma unroll
             for (int c = 0; c < 3; ++c) base[c] = f2_mul(f.gdm1, V[c]);
-            if (__any_sync(kFullMask, slow)) {
-                DriftFactors w;
-                const bool done = drift_wide_call(r2, sc.mudt, pc.dt, sc.dt, x, y, z, vx, vy, vz, w);
-                if (slow && done) {
-                    slow = false;
-                    f.fm1 = w.fm1;
-                    f.g = w.g;
-                    f.fd = w.fd;
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) base[c] = f2_muln(w.gdm1, f2_normp(V[c]));
-                }
-            }
             n[0] = fma(f.fm1, x, fma(f.g, vx, x));
             n[1] = fma(f.fm1, y, fma(f.g, vy, y));
             n[2] = fma(f.fm1, z, fma(f.g, vz, z));
@@ -297,6 +285,7 @@ __device__ __forceinline__ void advance_lane(const ParticleConsts& pc, const Spl
             n[5] = fma(f.fd, z, vz);
             if (__any_sync(kFullMask, slow)) {
                 double s[6] = {x, y, z, vx, vy, vz};
+                all_slow = __all_sync(kFullMask, slow || !act);
                 const bool done = drift_fp64(pc, slow, s);
                 if (slow) {
                     failed = !done;

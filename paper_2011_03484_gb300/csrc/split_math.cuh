@@ -101,16 +101,6 @@ __device__ __forceinline__ F2 f2_div(const F2& a, const F2& b, float rb) {
     return q;
 }
 
-// The same, normalised, to 2^-48.
-__device__ __forceinline__ F2 f2_divn(const F2& a, const F2& b, float rb) {
-    const float q = __fmul_rn(a.h, rb);
-    const float e = __fadd_rn(__fmaf_rn(-q, b.l, __fmaf_rn(-q, b.h, a.h)), a.l);
-    const float l = __fmul_rn(e, rb);
-    F2 r = f2_norm(q, l);
-    r.l = __fmaf_rn(__fmaf_rn(-l, b.h, e), rb, r.l);
-    return r;
-}
-
 // a - b c
 __device__ __forceinline__ F2 f2_fnma(const F2& b, const F2& c, const F2& a) { return f2_sub(a, f2_mul(b, c)); }
 
@@ -170,16 +160,6 @@ __device__ __forceinline__ F2 f2_dot(const F2 (&a)[3], const F2 (&b)[3]) {
     return s;
 }
 
-// f2_dot with normalised products.
-__device__ __forceinline__ F2 f2_dotn(const F2 (&a)[3], const F2 (&b)[3]) {
-    const F2 p = f2_muln(a[0], b[0]), q = f2_muln(a[1], b[1]), r = f2_muln(a[2], b[2]);
-    F2 s;
-    float e, f;
-    two_sum(p.h, q.h, s.h, e);
-    two_sum(s.h, r.h, s.h, f);
-    return f2_norm(s.h, __fadd_rn(__fadd_rn(e, f), __fadd_rn(__fadd_rn(p.l, q.l), r.l)));
-}
-
 // A double as a pair, by integer operations and one int-to-float conversion
 // (an F2F conversion occupies the FP64 pipe): the leading 24 bits, and the other
 // 29 rounded to 24.  |x| below 2^-74 is read as 2^-74 (1 + ...): far below
@@ -206,22 +186,6 @@ __device__ __forceinline__ double f21_square(float y) {
     const unsigned long long m2 = (unsigned long long)m * m;     // [2^40, 2^42)
     const int a = (int)(m2 >> 41);
     return __longlong_as_double(((long long)(2 * (int)(b >> 23) + 768 + a) << 52) + (long long)(m2 << (12 - a)));
-}
-
-// f2_split with the leading part rounded to nearest: the rest, and its rounding error,
-// are half as large (four instructions more).
-__device__ __forceinline__ F2 f2_split_near(double x) {
-    const unsigned lo = (unsigned)__double2loint(x), hi = (unsigned)__double2hiint(x);
-    const unsigned long long a =
-        ((unsigned long long)max(hi & 0x7FFFFFFFu, (unsigned)(1023 - 74) << 20) << 32) | lo;
-    const unsigned long long r = a + 0x10000000ull;
-    const unsigned sign = hi & 0x80000000u;
-    F2 v;
-    v.h = __uint_as_float((__funnelshift_l((unsigned)r, (unsigned)(r >> 32), 3) + 0x40000000u) | sign);
-    // the 29 low bits as a signed number, in units of 2^-55 of x's binade
-    const unsigned sc = ((((unsigned)(a >> 32) << 3) & 0xFF800000u) + 0x40000000u - (55u << 23)) | sign;
-    v.l = __fmul_rn((float)(int)(lo << 3), __uint_as_float(sc));
-    return v;
 }
 
 // k y^3 correctly rounded (ties away from zero) for a float y > 0 of at most 21 significant

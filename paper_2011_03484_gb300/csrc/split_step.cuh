@@ -7,8 +7,8 @@
 // One step then takes 19 FP64 instructions (r^2 and dt mu / r^3: 5; g, fdot: 2;
 // f x + g v: 6; fdot x: 3; gdot v and the kick, summed in pairs: 3) against 61 + 12 N_p for
 // the all-FP64 step, and ~1200 instructions in all, which fit under them.
-// Measured (1048576 particles, 4 planets, 1024 steps): 44.8 ms against 207 ms; the 19
-// instructions at 65 cycles are 73% of that.  Against 113-bit arithmetic, one step's velocity
+// Measured (1048576 particles, 4 planets, 1024 steps): 46.4 ms against 207 ms; the 19
+// instructions at 65 cycles are 71% of that.  Against 113-bit arithmetic, one step's velocity
 // is off by 0.58 to 0.71 units of 2^-53 (rms over belts of 20-100 AU; the all-FP64 step:
 // 1.09 to 1.21): fewer roundings, and what the pairs drop lies below them.
 #pragma once
@@ -48,7 +48,8 @@ __host__ __device__ inline void split_step_consts(const ParticleConsts& pc, Spli
 // are FP64.  S: series start, one Newton step in FP32, one in pairs (the error
 // left is below (a/2) (2^-18)^2).
 // Domain: |a| <= kSplitA, b and m <= kSplitZ; the caller runs the FP64 drift for
-// other lanes.
+// other lanes.  (A form of the pairs kept to 2^-48 for steps up to m = 3/64 took 7700 cycles for
+// a lone warp against the FP64 drift's 4500, and 15% more on orbits up to e = 0.9.)
 // ---------------------------------------------------------------------------
 constexpr float kSplitZ = 0.00390625f;  // 2^-8
 constexpr float kSplitA = 0.046875f;    // 3/64
@@ -65,6 +66,12 @@ __device__ __forceinline__ Speed float_speed(double r2, double vx, double vy, do
     const float a = d2f_bits(vx), b = d2f_bits(vy), c = d2f_bits(vz);
     const float v2 = fmaf(a, a, fmaf(b, b, c * c));
     return Speed{in_float_range(r2) ? v2 : -1.0f, __fdividef(v2, d2f_bits(r2))};
+}
+
+// True where m = mu dt^2 / r^3 alone puts a lane outside drift_split's domain.
+__device__ __forceinline__ bool beyond_split(double r2, float mudt, float dt) {
+    const float y = rsqrt_f32(f32_trunc(r2));
+    return in_float_range(r2) && mudt * dt * (y * y * y) > 1.001f * kSplitZ;
 }
 
 struct DriftFactors {
@@ -100,6 +107,15 @@ __device__ __forceinline__ void inverse_powers(double r2, double mudt, F2& w, do
     fast_two_sum(yy, p, w.h, e);
     w.l = __fadd_rn(__fadd_rn(e, __fmaf_rn(yy, er.h, -p)),
                     __fmaf_rn(yy, __fmaf_rn(er.h, er.h, er.l), __fmaf_rn(yl, er.h, yl)));
+}
+
+// drift_split's speed alone.
+__device__ __forceinline__ Speed split_speed(double r2, double mudt, const F2 (&v)[3]) {
+    F2 w;
+    double dts;
+    inverse_powers(r2, mudt, w, dts);
+    const F2 v2 = f2_dot(v, v);
+    return Speed{v2.h, v2.h * w.h};
 }
 
 // mudt = mu dt, dt2 = dt; ser (or null) receives the scalars.
@@ -196,143 +212,6 @@ __device__ __forceinline__ bool drift_split(double r2, double mudt, double dt, c
     out.gdm1 = gd;
     out.g = fma(-dt, f2_double(f2_norm(mg3.h, mg3.l)), dt);
     out.fd = fma(-dts, f2_double(f2_norm(k.h, k.l)), -dts);
-    return ok;
-}
-
-// ---------------------------------------------------------------------------
-// The drift for longer steps (m or b above kSplitZ, up to kWideZ: a planet-crossing
-// particle near its pericentre, a short-period system).  The corrections reach
-// 2^-4 there, so the pairs are kept to 2^-48 of their own values: products are
-// normalised (f2_muln), k, e2 = 2 g2 - 1 and 1/D - 1 are summed from small values
-// and never through a number near 1, S is a pair, and f - 1 starts from m in FP64:
-//   f - 1 = -(m/2) (1 + e2),  gdot - 1 = (f - 1) (1 + kd),  kd = 1/D - 1.
-// ~700 instructions and 2 FP64 ones more than drift_split, against ~63 FP64 ones for
-// the all-FP64 drift.  Its error is the FP64 drift's up to b = 0.015 (v 0.74 against
-// 0.65 units of 2^-53) and 0.99 against 0.67 at 0.03, where the kick's fewer roundings
-// still keep the step below the all-FP64 one; beyond, the FP64 drift.
-// ---------------------------------------------------------------------------
-constexpr float kWideZ = 0.046875f;  // 3/64
-constexpr float kWideA = 0.0625f;    // 2^-4
-
-// c + x y for |c| above |x y| (c: a constant's pair)
-__device__ __forceinline__ F2 f2_horner(const F2& c, const F2& x, const F2& y) {
-    const F2 p = f2_mul(x, y);
-    F2 r;
-    float e;
-    fast_two_sum(c.h, p.h, r.h, e);
-    r.l = __fadd_rn(__fadd_rn(e, c.l), p.l);
-    return r;
-}
-
-__device__ __forceinline__ bool drift_wide(double r2, double mudt, double dt, const F2& dt2, const double (&s)[6],
-                                           DriftFactors& out) {
-    F2 u, v2;
-    {
-        const F2 x[3] = {f2_split_near(s[0]), f2_split_near(s[1]), f2_split_near(s[2])};
-        const F2 v[3] = {f2_split_near(s[3]), f2_split_near(s[4]), f2_split_near(s[5])};
-        u = f2_dotn(x, v);
-        v2 = f2_dotn(v, v);
-    }
-    F2 w;
-    double dts;
-    inverse_powers(r2, mudt, w, dts);
-    const F2 dw = f2_muln(dt2, w);
-    const F2 a = f2_muln(u, dw);
-    const F2 n = f2_muln(v2, f2_muln(dt2, dw));
-    const double md = dt * dts;
-    const F2 m = f2_split(md);
-    const F2 q = f2_sub(n, m);
-    const F2 b = f2_sub(m, q);
-
-    // ---- S in FP32 ----
-    float S = __fmaf_rn(-1.0f / 6.0f, q.h, __fmaf_rn(0.5f * a.h, a.h - 1.0f, 1.0f));
-#pragma unroll
-    for (int it = 0; it < 3; ++it) {
-        const float s2 = S * S, z = b.h * s2;
-        const float g2 = s2 * __fmaf_rn(z, __fmaf_rn(z, __fmaf_rn(z, -1.0f / 40320.0f, 1.0f / 720.0f), -1.0f / 24.0f),
-                                        0.5f);
-        const float g3 = s2 * S * __fmaf_rn(z, __fmaf_rn(z, 1.0f / 5040.0f, -1.0f / 120.0f), 1.0f / 6.0f);
-        const float F = __fmaf_rn(a.h, g2, __fmaf_rn(q.h, g3, S - 1.0f));
-        const float D = __fmaf_rn(q.h, g2, __fmaf_rn(a.h, 1.0f - __fmaf_rn(a.h, g2, m.h * g3), 1.0f));
-        S = __fmaf_rn(-F, rcp_f32(D), S);
-    }
-    // ---- at S: 2 g2 = (1 + sm)(1 + t2) = 1 + e2,  6 g3 = S^3 (1 + t3) ----
-    F2 s2, s3;
-    s2.h = __fmul_rn(S, S);
-    s2.l = __fmaf_rn(S, S, -s2.h);
-    s3.h = __fmul_rn(s2.h, S);
-    s3.l = __fmaf_rn(s2.l, S, __fmaf_rn(s2.h, S, -s3.h));
-    const F2 z = f2_muln(b, s2);
-    const float zh = z.h;
-    // t2 = z (-1/12 + z/360 - z^2/20160 + z^3/1814400 - ...), t3 = z (-1/20 + z/840 - z^2/60480 + ...)
-    constexpr F2 p21 = {-0.083333336f, 2.483527e-09f}, p22 = {0.0027777778f, -6.726219e-11f},
-                 p23 = {-4.9603175e-05f, 6.813992e-13f};
-    constexpr F2 p31 = {-0.05f, 7.4505807e-10f}, p32 = {0.0011904762f, -4.5457412e-11f};
-    F2 t2, t3;
-    {
-        const float y2 = zh * __fmaf_rn(zh, __fmaf_rn(zh, 2.294149e-11f, -4.175351e-09f), 5.511464e-07f);
-        F2 h2;
-        fast_two_sum(p23.h, y2, h2.h, h2.l);
-        h2.l = __fadd_rn(h2.l, p23.l);
-        t2 = f2_muln(z, f2_horner(p21, z, f2_horner(p22, z, h2)));
-        const float y3 = zh * __fmaf_rn(zh, __fmaf_rn(zh, -9.635426e-10f, 1.5031264e-07f), -1.6534392e-05f);
-        F2 h3;
-        fast_two_sum(p32.h, y3, h3.h, h3.l);
-        h3.l = __fadd_rn(h3.l, p32.l);
-        t3 = f2_muln(z, f2_horner(p31, z, h3));
-    }
-    const F2 sm = f2_norm(__fsub_rn(s2.h, 1.0f), s2.l);
-    F2 e2 = f2_add(f2_add(sm, t2), f2_mul(sm, t2));
-    F2 g3 = f2_mul(s3, t3);  // 6 g3 = s3 + s3 t3
-    {
-        float t;
-        fast_two_sum(s3.h, g3.h, g3.h, t);
-        g3.l = __fadd_rn(t, __fadd_rn(s3.l, g3.l));
-    }
-    const F2 a2 = {0.5f * a.h, 0.5f * a.l}, q2 = {0.5f * q.h, 0.5f * q.l};
-    constexpr F2 k6 = {0.16666667f, -4.967054e-09f};
-    const F2 q6 = f2_muln(q, k6), m6 = f2_muln(m, k6);
-    const F2 ag = f2_add(a2, f2_mul(a2, e2));   // a g2
-    const F2 qg = f2_add(q2, f2_mul(q2, e2));   // q g2
-    const F2 q3 = f2_mul(q6, g3), m3 = f2_mul(m6, g3);  // q g3, m g3
-    const F2 S1 = {__fsub_rn(S, 1.0f), 0.0f};
-    // F = (S - 1) + a g2 + q g3; y1 = g1 - 1 = (S - 1) - b g3; rho = D - 1 = a + a y1 + q g2
-    const F2 F = f2_normp(f2_add(f2_add(S1, ag), q3));
-    const F2 y1 = f2_add(f2_sub(S1, m3), q3);
-    F2 rho = f2_add(f2_add(a, f2_mul(a, y1)), qg);
-    // d = -F / D as a pair
-    const float rD0 = rcp_f32(__fadd_rn(1.0f, rho.h));
-    F2 d;
-    d.h = __fmul_rn(-F.h, rD0);
-    // residual F + d D = (F.h + d.h) + F.l + d.h rho
-    d.l = __fmul_rn(__fadd_rn(__fadd_rn(F.h, d.h), __fmaf_rn(d.h, rho.h, F.l)), -rD0);
-    const bool ok = fabsf(a.h) <= kWideA && fabsf(b.h) <= kWideZ && m.h <= kWideZ && fabsf(d.h) <= 3.8146973e-6f;
-    // to S + d (second order in d included): g2 + d g1 + d^2 g0 / 2, g3 + d g2, y1 + d g0, D + d (a g0 + q g1)
-    const float g0f = __fmaf_rn(-b.h, __fmaf_rn(0.5f, e2.h, 0.5f), 1.0f), g1f = __fadd_rn(1.0f, y1.h);
-    const float dy = __fmaf_rn(0.5f * d.h, g0f, y1.h);  // g1 - 1 halfway
-    const F2 dg2 = f2_norm(d.h, __fmaf_rn(d.h, dy, d.l));  // g2(S + d) - g2
-    e2 = f2_add(e2, F2{2.0f * dg2.h, 2.0f * dg2.l});
-    const float dg3 = d.h * __fmaf_rn(0.5f * d.h, g1f, __fmaf_rn(0.5f, e2.h, 0.5f));
-    const F2 mg3 = f2_add(m3, F2{m.h * dg3, 0.0f});
-    const F2 T = f2_add(f2_add(a2, f2_mul(a2, e2)), mg3);  // a g2 + m g3 = 1 - g1
-    rho = f2_normp(f2_add(f2_sub(a, f2_mul(a, T)), f2_add(q2, f2_mul(q2, e2))));
-    F2 N = f2_add(T, rho);
-    N = f2_norm(-N.h, -N.l);  // g1 - D
-    F2 D;
-    fast_two_sum(1.0f, rho.h, D.h, D.l);
-    D.l = __fadd_rn(D.l, rho.l);
-    const float rD = rcp_f32(D.h);
-    const F2 k = f2_divn(N, D, rD), kd = f2_divn(F2{-rho.h, -rho.l}, D, rD);
-    const double mh = -0.5 * md;
-    out.fm1 = fma(mh, f2_double(f2_normp(e2)), mh);
-    F2 e1, kd1;  // 1 + e2, 1 + kd
-    fast_two_sum(1.0f, e2.h, e1.h, e1.l);
-    e1.l = __fadd_rn(e1.l, e2.l);
-    fast_two_sum(1.0f, kd.h, kd1.h, kd1.l);
-    kd1.l = __fadd_rn(kd1.l, kd.l);
-    out.gdm1 = f2_muln(f2_muln(F2{-0.5f * m.h, -0.5f * m.l}, f2_normp(e1)), f2_normp(kd1));
-    out.g = fma(-dt, f2_double(f2_normp(mg3)), dt);
-    out.fd = fma(-dts, f2_double(k), -dts);
     return ok;
 }
 
