@@ -66,15 +66,6 @@ __device__ __forceinline__ F2 f2_mul(const F2& a, const F2& b) {
     return r;
 }
 
-// Product, normalised, of normalised pairs: to 2^-48.
-__device__ __forceinline__ F2 f2_muln(const F2& a, const F2& b) {
-    const float h = __fmul_rn(a.h, b.h);
-    const float t = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmul_rn(a.l, b.l)));
-    return f2_norm(h, __fadd_rn(__fmaf_rn(a.h, b.h, -h), t));
-}
-
-__device__ __forceinline__ F2 f2_normp(const F2& a) { return f2_norm(a.h, a.l); }
-
 __device__ __forceinline__ F2 f2_add(const F2& a, const F2& b) {
     F2 r;
     float e;
